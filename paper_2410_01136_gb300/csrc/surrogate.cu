@@ -7,10 +7,11 @@
 // HEALPix pixels: e_i[p] = s_p H_N[r_i, p] / sqrt(N), with seeded signs s_p,
 // seeded distinct rows r_i and H_N = H_12 (x) H_M (M = Nside^2) the Kronecker
 // product of Paley's Hadamard matrix of order 12 and Sylvester's of order M.
-// The +-1 matrix s_p H_N[r_i, p] is exact in BF16; a map m (FP32) is split
-// as m = hi + lo with both halves BF16, so the projection
-// c = (S hi + S lo) / sqrt(N) runs as two tensor-core GEMMs with FP32
-// accumulation and loses only the 2^-17 relative split residual.
+// The projection is a fast Walsh-Hadamard transform in FP32 (srht.cu); no
+// matrix is formed.  The basis of spherical harmonics (sh_basis.cu) is dense:
+// there a map m (FP32) is split as m = hi + lo with both halves BF16 and
+// projected by tensor-core GEMMs with FP32 accumulation, which lose only the
+// 2^-17 relative split residual.
 //
 // Network.  theta -> x = 2 (theta - lo) / (hi - lo) - 1 (padded to 64
 // inputs with zeros) -> depth hidden layers of `width` with GELU -> the
@@ -44,6 +45,7 @@
 #include <vector>
 
 #include "gemm.cuh"
+#include "srht.cuh"
 #include "synax_internal.h"
 
 using bf16 = __nv_bfloat16;
@@ -59,8 +61,6 @@ constexpr int kInPad = 64;             // network inputs padded to one K tile
 constexpr int kLossHist = 1 << 16;     // device ring of per-step losses
 constexpr uint32_t kMagic = 0x53555253u;   // "SRUS"
 constexpr uint32_t kFileVersion = 1;
-
-__constant__ int8_t c_h12[144];
 
 // Paley's construction of a Hadamard matrix of order 12 over GF(11):
 // H = I + [[0, 1^T], [-1, Q]], Q[i][j] = chi(j - i), chi the quadratic
@@ -85,21 +85,6 @@ void paley12(int8_t* H) {
 // ---------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------
-
-// S[i][p] = sign[p] * H_12[r_i / M][p / M] * (-1)^popcount((r_i % M) & (p % M))
-__global__ void k_build_basis(bf16* __restrict__ S, const int8_t* __restrict__ sign, const int* __restrict__ rows,
-                              int n_basis, int npix, int M) {
-    const long long total = (long long)n_basis * npix;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(e / npix);
-        const int p = (int)(e - (long long)i * npix);
-        const int r = rows[i];
-        int h = c_h12[(r / M) * 12 + p / M] * sign[p];
-        if (__popc((unsigned)((r % M) & (p % M))) & 1) h = -h;
-        S[e] = __float2bfloat16_rn((float)h);
-    }
-}
 
 // m = hi + lo, hi = bf16(m), lo = bf16(m - hi)
 __global__ void k_split_hi_lo(const float* __restrict__ m, long long n, bf16* __restrict__ hi, bf16* __restrict__ lo) {
@@ -508,11 +493,10 @@ struct synax_surrogate_s {
     float* eZ[kMaxLayers] = {nullptr};
     bf16 *eD0 = nullptr, *eD1 = nullptr;
     // basis and map staging
-    int8_t* sign_dev = nullptr;
+    uint32_t* sign_dev = nullptr;   // SRHT: one sign bit per pixel
     int* basis_rows_dev = nullptr;
-    bf16* S = nullptr;
-    bf16* S_lo = nullptr;       // basis_kind 1: the basis' BF16 low part (E = S + S_lo)
-    float proj_scale = 1.0f;    // coefficient = proj_scale * (S x): 1/sqrt(npix) for the +-1 basis
+    bf16* S = nullptr;              // SH: the dense basis as BF16 hi + lo (E = S + S_lo)
+    bf16* S_lo = nullptr;
     float* maps = nullptr;
     bf16 *mhi = nullptr, *mlo = nullptr;
     float* ctrue = nullptr;
@@ -669,21 +653,29 @@ GatherArgs gather_identity(const synax_surrogate_t* s, const float* theta, int c
     return a;
 }
 
-// Coefficients of `rows` maps already split into s->mhi + s->mlo:
-// out = proj_scale (S_hi x_hi + S_hi x_lo [+ S_lo x_hi for basis_kind 1]).
-int project_split(synax_surrogate_t* s, int rows, float* out, cudaStream_t st) {
+// Coefficients of `rows` maps (at most 3 * chunk of them): the fast transform
+// of the SRHT basis, or for the SH basis the split maps against its BF16
+// hi + lo rows, out = S x_hi + S x_lo + S_lo x_hi.
+int project_rows(synax_surrogate_t* s, const float* maps, int rows, float* out, cudaStream_t st) {
+    if (s->cfg.basis_kind == SYNAX_SUR_BASIS_SRHT) {
+        int lg = 0;
+        while ((1 << lg) < s->cfg.nside) ++lg;
+        const SrhtBasis B{2 * lg, s->cfg.n_basis, (float)(1.0 / std::sqrt((double)s->npix)), s->sign_dev,
+                          s->basis_rows_dev};
+        return srht_project(B, maps, rows, out, st);
+    }
+    const long long n = (long long)rows * s->npix;
+    k_split_hi_lo<<<grid_for(n), 256, 0, st>>>(maps, n, s->mhi, s->mlo);
+    SX_TRY(launch_status());
     GemmEpiParams ep{};
     ep.out_f32 = out;
     ep.ld_f32 = s->cfg.n_basis;
-    ep.scale = s->proj_scale;
+    ep.scale = 1.0f;
     ep.accumulate = 0;
     SX_TRY(gemm_bf16(s->mhi, s->npix, s->S, s->npix, rows, s->cfg.n_basis, s->npix, EPI_SCALE_ACC, ep, s->err, st));
     ep.accumulate = 1;
     SX_TRY(gemm_bf16(s->mlo, s->npix, s->S, s->npix, rows, s->cfg.n_basis, s->npix, EPI_SCALE_ACC, ep, s->err, st));
-    if (s->S_lo)
-        SX_TRY(gemm_bf16(s->mhi, s->npix, s->S_lo, s->npix, rows, s->cfg.n_basis, s->npix, EPI_SCALE_ACC, ep, s->err,
-                         st));
-    return SYNAX_OK;
+    return gemm_bf16(s->mhi, s->npix, s->S_lo, s->npix, rows, s->cfg.n_basis, s->npix, EPI_SCALE_ACC, ep, s->err, st);
 }
 
 // Render `count` maps of the fiducial problem at theta_host rows into
@@ -696,10 +688,7 @@ int render_and_project(synax_surrogate_t* s, const synax_problem* fid, const dou
         for (int j = 0; j < nt; ++j) P.theta[j] = theta_host[(long long)k * nt + j];
         SX_TRY(synax_forward(&P, s->maps + (long long)k * 3 * s->npix, st));
     }
-    const long long n = (long long)count * 3 * s->npix;
-    k_split_hi_lo<<<grid_for(n), 256, 0, st>>>(s->maps, n, s->mhi, s->mlo);
-    SX_TRY(launch_status());
-    return project_split(s, 3 * count, out, st);
+    return project_rows(s, s->maps, 3 * count, out, st);
 }
 
 int check_fiducial(const synax_surrogate_t* s, const synax_problem* fid) {
@@ -788,11 +777,9 @@ int synax_surrogate_create(const synax_surrogate_cfg* cfg, synax_surrogate_t** o
     if (c.basis_kind == SYNAX_SUR_BASIS_SRHT) {
         s->sign.assign(c.basis_sign, c.basis_sign + npix);
         s->rows.assign(c.basis_rows, c.basis_rows + c.n_basis);
-        s->proj_scale = (float)(1.0 / std::sqrt((double)npix));
     } else {
         s->sign.assign(npix, 0);
         s->rows.assign(c.n_basis, 0);
-        s->proj_scale = 1.0f;
     }
     s->npix = npix;
     s->n_out = 3 * c.n_basis;
@@ -835,11 +822,14 @@ int synax_surrogate_create(const synax_surrogate_cfg* cfg, synax_surrogate_t** o
     s->n_part = gemm_tiles(B, s->n_out, c.width);
     SX_ALLOC(s->loss_part, s->n_part) SX_ALLOC(s->loss_hist, kLossHist)
     SX_ALLOC(s->t_dev, 1) SX_ALLOC(s->adam_coef, 4) SX_ALLOC(s->err, 1)
-    SX_ALLOC(s->sign_dev, npix) SX_ALLOC(s->basis_rows_dev, c.n_basis)
-    SX_ALLOC(s->S, (long long)c.n_basis * npix)
-    if (c.basis_kind == SYNAX_SUR_BASIS_SH) SX_ALLOC(s->S_lo, (long long)c.n_basis * npix)
+    std::vector<uint32_t> sign_words;
+    srht_pack_signs(s->sign.data(), npix, sign_words);
+    SX_ALLOC(s->sign_dev, sign_words.size()) SX_ALLOC(s->basis_rows_dev, c.n_basis)
+    if (c.basis_kind == SYNAX_SUR_BASIS_SH) {
+        SX_ALLOC(s->S, (long long)c.n_basis * npix) SX_ALLOC(s->S_lo, (long long)c.n_basis * npix)
+        SX_ALLOC(s->mhi, (long long)s->chunk * 3 * npix) SX_ALLOC(s->mlo, (long long)s->chunk * 3 * npix)
+    }
     SX_ALLOC(s->maps, (long long)s->chunk * 3 * npix)
-    SX_ALLOC(s->mhi, (long long)s->chunk * 3 * npix) SX_ALLOC(s->mlo, (long long)s->chunk * 3 * npix)
     SX_ALLOC(s->ctrue, (long long)s->chunk * s->n_out)
 #undef SX_ALLOC
     // zero weights and state; basis; normalisation of inputs and outputs
@@ -859,9 +849,9 @@ int synax_surrogate_create(const synax_surrogate_cfg* cfg, synax_surrogate_t** o
     if (e == cudaSuccess) e = cudaMemset(s->err, 0, 4);
     if (e == cudaSuccess) e = cudaMemcpy(s->lo, lo_h, sizeof lo_h, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(s->inv2, inv2_h, sizeof inv2_h, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->sign_dev, s->sign.data(), npix, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(s->sign_dev, sign_words.data(), 4 * sign_words.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(s->basis_rows_dev, s->rows.data(), 4 * (size_t)c.n_basis, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_h12, h12, sizeof h12);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming);
@@ -869,9 +859,7 @@ int synax_surrogate_create(const synax_surrogate_cfg* cfg, synax_surrogate_t** o
     if (e != cudaSuccess) return fail(record_cuda_error((int)e));
     if ((rc = gemm_init()) != SYNAX_OK) return fail(rc);
     if (c.basis_kind == SYNAX_SUR_BASIS_SRHT) {
-        k_build_basis<<<grid_for((long long)c.n_basis * npix), 256>>>(s->S, s->sign_dev, s->basis_rows_dev, c.n_basis,
-                                                                       npix, c.nside * c.nside);
-        if ((rc = launch_status()) != SYNAX_OK) return fail(rc);
+        if ((rc = srht_init(h12)) != SYNAX_OK) return fail(rc);
     } else if ((rc = build_sh_basis(c.nside, c.n_basis, s->S, s->S_lo, nullptr)) != SYNAX_OK) {
         return fail(rc);
     }
@@ -996,10 +984,7 @@ int synax_surrogate_project(synax_surrogate_t* s, const float* maps_dev, long lo
     const long long cap = 3LL * s->chunk;
     for (long long r0 = 0; r0 < n_rows; r0 += cap) {
         const int rows = (int)(n_rows - r0 < cap ? n_rows - r0 : cap);
-        const long long n = (long long)rows * s->npix;
-        k_split_hi_lo<<<grid_for(n), 256, 0, st>>>(maps_dev + r0 * s->npix, n, s->mhi, s->mlo);
-        SX_TRY(launch_status());
-        SX_TRY(project_split(s, rows, coeffs_dev + r0 * s->cfg.n_basis, st));
+        SX_TRY(project_rows(s, maps_dev + r0 * s->npix, rows, coeffs_dev + r0 * s->cfg.n_basis, st));
     }
     return SYNAX_OK;
 }
