@@ -4,7 +4,8 @@
 // copies).
 //
 // Persistent and warp-specialised: min(tiles, SMs) CTAs (192 threads, or 320
-// for the GELU, GELU' and MSE epilogues, which get 8 epilogue warps) walk
+// for the GELU, GELU' and MSE epilogues of tiles wider than 32 columns, which
+// get 8 epilogue warps) walk
 // the 128 x BN output tiles (row-major tile order, so concurrent CTAs share
 // A row blocks and the whole B operand stays in L2):
 //   warp 0 (one thread)  TMA producer: a ring of ST stages, each a 128x64 A
@@ -53,14 +54,15 @@ constexpr int kGemmBK = 64;
 // row per thread) are latency-bound with one warp per scheduler, so they get
 // 8 warps, two per TMEM lane quadrant, each taking half of the tile's
 // columns; the FP32 epilogues keep 4, one per quadrant, which their TMA-store
-// staging chunks (128 rows x 32 columns) are laid out for.
-template <int EPI>
+// staging chunks (128 rows x 32 columns) are laid out for, and so do 32-column
+// tiles, which are one block wide.
+template <int BN, int EPI>
 constexpr int gemm_epi_warps() {
-    return EPI == EPI_BIAS_GELU || EPI == EPI_GELU_BWD || EPI == EPI_MSE ? 8 : 4;
+    return BN > 32 && (EPI == EPI_BIAS_GELU || EPI == EPI_GELU_BWD || EPI == EPI_MSE) ? 8 : 4;
 }
-template <int EPI>
+template <int BN, int EPI>
 constexpr int gemm_threads() {
-    return 64 + 32 * gemm_epi_warps<EPI>();
+    return 64 + 32 * gemm_epi_warps<BN, EPI>();
 }
 constexpr long long kWaitCycles = 2000000000LL;   // ~1 s at 2 GHz
 
@@ -247,7 +249,7 @@ __device__ __forceinline__ void epilogue16(const GemmEpiParams& ep, const float*
 }
 
 template <int BN, int EPI>
-__global__ void __launch_bounds__(gemm_threads<EPI>(), 1)
+__global__ void __launch_bounds__(gemm_threads<BN, EPI>(), 1)
 k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
             const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmD, int M, int N, int K,
             GemmEpiParams ep, int* err) {
@@ -265,7 +267,7 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     uint64_t* acc_empty = acc_full + 2;   // [2]
     uint64_t* drain = acc_empty + 2;
     uint32_t* tmem_slot = (uint32_t*)(drain + 1);
-    constexpr int EW = gemm_epi_warps<EPI>();
+    constexpr int EW = gemm_epi_warps<BN, EPI>();
     __shared__ float red[8];
 
     const int warp = threadIdx.x >> 5;
@@ -588,11 +590,25 @@ __global__ void __launch_bounds__(64, 1) k_wait_selftest(int* err, long long* cy
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-// tile width: 256 for wide outputs, and for medium ones with a long K (the A
-// row block is then re-read by half as many column tiles and each stage
-// feeds twice the MMA work); 128 for medium, 64 for narrow ones
-static int gemm_bn_for(int N, int K) {
-    return (N >= 2048 || (N >= 1024 && K >= 4096)) ? 256 : (N >= 256 ? 128 : 64);
+// Tile width.  With tiles for every SM: 256 for wide outputs, and for medium
+// ones with a long K (the A row block is then re-read by half as many column
+// tiles and each stage feeds twice the MMA work); 128 for medium, 64 for
+// narrow ones.
+// Few rows leave SMs without a tile, and a tile's time is then the operand
+// bytes that its SM takes in, 128 (128 + BN) per K tile (about 60 B per clock:
+// a 128 x 256 tile at K = 9216 took 62 us on 4 to 16 SMs).  Halving the width
+// is taken while it lowers waves x bytes, so that the same product runs as
+// narrower tiles on more SMs: 512 x 1024 x 9216 60.5 -> 44.2 us and 512 x 1024
+// x 1024 15.6 -> 11.0 us (32 columns, 128 tiles).  The order of summation
+// along K does not depend on the width.
+static int gemm_bn_for(int M, int N, int K, int sms) {
+    int bn = (N >= 2048 || (N >= 1024 && K >= 4096)) ? 256 : (N >= 256 ? 128 : 64);
+    auto cost = [&](int w) {
+        const long long tiles = (long long)((N + w - 1) / w) * ((M + kGemmBM - 1) / kGemmBM);
+        return (tiles + sms - 1) / sms * (kGemmBM + w);
+    };
+    while (bn > 32 && cost(bn / 2) < cost(bn)) bn /= 2;
+    return bn;
 }
 
 namespace {
@@ -649,7 +665,8 @@ cudaError_t set_smem_attr() {
 
 template <int EPI>
 cudaError_t set_smem_attrs() {
-    cudaError_t e = set_smem_attr<64, EPI>();
+    cudaError_t e = set_smem_attr<32, EPI>();
+    if (e == cudaSuccess) e = set_smem_attr<64, EPI>();
     if (e == cudaSuccess) e = set_smem_attr<128, EPI>();
     if (e == cudaSuccess) e = set_smem_attr<256, EPI>();
     return e;
@@ -710,7 +727,7 @@ int launch_gemm_t(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, in
     if (GemmCfg<BN, EPI>::BF16_STAGE && ep.out_bf16 && !ep.out_bf16_t && ((uintptr_t)ep.out_bf16 & 15) == 0 &&
         (ep.ld_bf16 & 7) == 0 && make_bf16_out_map(&md, ep.out_bf16, M, N, ep.ld_bf16) == SYNAX_OK)
         ep.tma_store_bf16 = 1;
-    k_gemm_bf16<BN, EPI><<<grid, gemm_threads<EPI>(), GemmCfg<BN, EPI>::SMEM, st>>>(ma, mb, mc, md, M, N, K, ep,
+    k_gemm_bf16<BN, EPI><<<grid, gemm_threads<BN, EPI>(), GemmCfg<BN, EPI>::SMEM, st>>>(ma, mb, mc, md, M, N, K, ep,
                                                                                        err);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SYNAX_OK : record_cuda_error((int)e);
@@ -720,7 +737,7 @@ template <int EPI>
 int launch_gemm_bn(const CUtensorMap& ma, const void* B, int N, int K, int ldb, int M, const GemmEpiParams& ep,
                    int* err, cudaStream_t st) {
     CUtensorMap mb;
-    int bn = gemm_bn_for(N, K);
+    int bn = gemm_bn_for(M, N, K, sm_count());
     // FP32 outputs (their 128-row staging chunks keep the epilogue light): a
     // 128 x 256 tile fetches 768 KB of operands per 2 x 128 x 256 x K flop
     // against 512 KB per half the work at 128 columns, and the SMs' operand
@@ -739,8 +756,12 @@ int launch_gemm_bn(const CUtensorMap& ma, const void* B, int N, int K, int ldb, 
         if (make_map(&mb, B, N, K, ldb, 128) != SYNAX_OK) return SYNAX_EINVAL;
         return launch_gemm_t<128, EPI>(ma, mb, M, N, K, ep, err, st);
     }
-    if (make_map(&mb, B, N, K, ldb, 64) != SYNAX_OK) return SYNAX_EINVAL;
-    return launch_gemm_t<64, EPI>(ma, mb, M, N, K, ep, err, st);
+    if (bn == 64) {
+        if (make_map(&mb, B, N, K, ldb, 64) != SYNAX_OK) return SYNAX_EINVAL;
+        return launch_gemm_t<64, EPI>(ma, mb, M, N, K, ep, err, st);
+    }
+    if (make_map(&mb, B, N, K, ldb, 32) != SYNAX_OK) return SYNAX_EINVAL;
+    return launch_gemm_t<32, EPI>(ma, mb, M, N, K, ep, err, st);
 }
 
 }  // namespace
@@ -765,7 +786,7 @@ int gemm_init() {
 int device_sm_count() { return sm_count(); }
 
 int gemm_tiles(int M, int N, int K) {
-    const int bn = gemm_bn_for(N, K);
+    const int bn = gemm_bn_for(M, N, K, sm_count());
     const int tiles = ((N + bn - 1) / bn) * ((M + kGemmBM - 1) / kGemmBM);
     return tiles < sm_count() ? tiles : sm_count();
 }
