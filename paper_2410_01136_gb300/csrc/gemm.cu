@@ -272,6 +272,10 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    // The set-up below touches no global memory, so it may run while the
+    // previous kernel of the stream finishes, and the next one's while this
+    // one runs (every CTA of this grid is resident by then).
+    tc::launch_dependents();
     if (threadIdx.x == 0) {
         tc::prefetch_tmap(&tmA);
         tc::prefetch_tmap(&tmB);
@@ -291,6 +295,7 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    tc::grid_dependency_wait();
 
     const int tiles_n = (N + BN - 1) / BN;
     const int tiles = tiles_n * ((M + kGemmBM - 1) / kGemmBM);
@@ -727,9 +732,18 @@ int launch_gemm_t(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, in
     if (GemmCfg<BN, EPI>::BF16_STAGE && ep.out_bf16 && !ep.out_bf16_t && ((uintptr_t)ep.out_bf16 & 15) == 0 &&
         (ep.ld_bf16 & 7) == 0 && make_bf16_out_map(&md, ep.out_bf16, M, N, ep.ld_bf16) == SYNAX_OK)
         ep.tma_store_bf16 = 1;
-    k_gemm_bf16<BN, EPI><<<grid, gemm_threads<BN, EPI>(), GemmCfg<BN, EPI>::SMEM, st>>>(ma, mb, mc, md, M, N, K, ep,
-                                                                                       err);
-    const cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)gemm_threads<BN, EPI>());
+    cfg.dynamicSmemBytes = GemmCfg<BN, EPI>::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = ep.overlap ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_bf16<BN, EPI>, ma, mb, mc, md, M, N, K, ep, err);
+    if (e == cudaSuccess) e = cudaGetLastError();
     return e == cudaSuccess ? SYNAX_OK : record_cuda_error((int)e);
 }
 

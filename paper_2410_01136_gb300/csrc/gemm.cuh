@@ -52,6 +52,8 @@ struct GemmEpiParams {
     int accumulate;              // EPI_SCALE_ACC
     int tma_store;               // set by gemm_bf16: FP32 output written through TMA stores
     int tma_store_bf16;          // set by gemm_bf16: GELU / GELU' BF16 output written through TMA stores
+    int overlap;                 // the stream's previous operation is a kernel of this library that this
+                                 // product may overlap with its own set-up (programmatic dependent launch)
     int* status;                 // set by gemm_bf16: the device status word (a timed-out wait reports there)
 };
 

@@ -47,6 +47,7 @@
 #include "gemm.cuh"
 #include "srht.cuh"
 #include "synax_internal.h"
+#include "tcgen05.cuh"
 
 using bf16 = __nv_bfloat16;
 
@@ -158,6 +159,7 @@ struct GatherArgs {
 __global__ void k_gather_input(GatherArgs a) {
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    tc::launch_dependents();
     if (b >= a.B) return;
     uint32_t src = (uint32_t)b;
     if (a.n) {
@@ -1141,6 +1143,7 @@ int synax_surrogate(synax_surrogate_t* s, const float* theta_dev, int n, float* 
         SX_TRY(launch_status());
         for (int l = 0; l < L; ++l) {
             GemmEpiParams ep{};
+            ep.overlap = 1;
             ep.bias = s->b + s->boff[l];
             if (l < L - 1) {
                 ep.out_z = vjp ? s->eZ[l] : nullptr;
@@ -1167,6 +1170,7 @@ int synax_surrogate(synax_surrogate_t* s, const float* theta_dev, int n, float* 
         bf16* d2 = s->eD1;
         for (int l = L - 1; l > 0; --l) {
             GemmEpiParams eb{};
+            eb.overlap = l < L - 1;      // the first one follows the side stream's join
             eb.aux = s->eZ[l - 1];
             eb.ld_aux = s->N[l - 1];
             eb.out_bf16 = d2;
@@ -1178,6 +1182,7 @@ int synax_surrogate(synax_surrogate_t* s, const float* theta_dev, int n, float* 
             d2 = tmp;
         }
         GemmEpiParams eo{};
+        eo.overlap = 1;
         eo.colscale = s->inv2;
         eo.out_f32 = gtheta_dev + (long long)r0 * nt;
         eo.ld_f32 = nt;
