@@ -18,7 +18,10 @@ constexpr int kAdjMinBlocks = 5;
 // node-gradient sums (48 registers), and the FP32 JF12-type one two samples'
 // field intermediates: 4 CTAs per SM leave them 128 registers (JF12-type map
 // + gradient 0.604 ms against 0.624 ms at 5 CTAs, where 264 bytes spilled).
-template <int MODEL> constexpr int adj_min_blocks() {
+// FP64 needs as many registers again: 3 per SM (168 registers; JF12-type map +
+// gradient at Nside 16, 100 steps, 3 frequencies 0.879 ms against 0.902 at 4).
+template <int MODEL, typename R> constexpr int adj_min_blocks() {
+    if (sizeof(R) == 8) return 3;
     return MODEL == SYNAX_MODEL_GRID || MODEL == SYNAX_MODEL_JF12 || MODEL == SYNAX_MODEL_WMAP ? 4 : kAdjMinBlocks;
 }
 
@@ -201,7 +204,9 @@ struct GridAcc {
         const R gz[2] = {R(1) - L.gfz, L.gfz};
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            const R wq = gx[q & 1] * gy[(q >> 1) & 1] * gz[(q >> 2) & 1];
+            R wq;
+            if constexpr (sizeof(R) == 8) wq = L.gw[q];
+            else wq = gx[q & 1] * gy[(q >> 1) & 1] * gz[(q >> 2) & 1];
             w[q][0] = fma(wq, bxb, w[q][0]);
             w[q][1] = fma(wq, byb, w[q][1]);
             w[q][2] = fma(wq, bzb, w[q][2]);
@@ -544,7 +549,7 @@ __device__ __forceinline__ void adjoint_cta(const MapParams<R>& P, const AdjPara
             if constexpr (sizeof(R) == 4) fzr = flat_z_of(P, nd);
             R nh = R(n1 - 1) + R(0.5);                  // n + 1/2, exact
             for (int n = n1 - 1; n >= n0; --n, nh -= R(1)) {
-                const R t = fma(nh, dr, nh * dr_lo);
+                const R t = sizeof(R) == 8 ? nh * dr : fma(nh, dr, nh * dr_lo);   // (as the forward march)
                 R x, y, z;
                 sample_pos<MODEL, R>(P, L, nd, t, x, y, z);
                 R B[3], N0, ne;
@@ -566,8 +571,9 @@ __device__ __forceinline__ void adjoint_cta(const MapParams<R>& P, const AdjPara
                 R bn, bb;
                 dot_n_eb<R>(B, L, bn, bb);
                 const R ba = B[0] * L.el[0] + B[1] * L.el[1];
-                const R bp2 = ba * ba + bb * bb;
-                const bool lit = bp2 > R(1e-30);
+                const R ba2 = ba * ba, bb2 = bb * bb;
+                const R bp2 = sizeof(R) == 8 ? ba2 + bb2 : ba * ba + bb * bb;
+                const bool lit = is_lit<R>(bp2);
                 const R lg = lit ? F::log2_fast(bp2) : R(0);
                 const R w = lit ? F::exp2_fast(q * lg) : R(0);
                 const R nw = N0 * w;
@@ -579,8 +585,8 @@ __device__ __forceinline__ void adjoint_cta(const MapParams<R>& P, const AdjPara
                     pc = v.x;
                     ps = v.y;
                 } else {
-                    pc = nw * (ba * ba - bb * bb);
-                    ps = nw * (R(2) * ba * bb);
+                    pc = nw * (ba2 - bb2);
+                    ps = (nw + nw) * (ba * bb);
                 }
                 R f = -ne * bn;
                 // as in the forward march (same operations, same rounding)
@@ -592,7 +598,7 @@ __device__ __forceinline__ void adjoint_cta(const MapParams<R>& P, const AdjPara
                 if constexpr (sizeof(R) == 4) {
                     ff_add_f_pair(Q, make_float2((P.w_own - 1.0f) * f, -f), s_n, Q);
                 } else {
-                    s_n = Ph::add(Q, (P.w_own - R(1)) * f);
+                    s_n = fma(P.w_own - R(1), f, Q);
                     Q = Ph::add(Q, -f);
                 }
                 R Or = R(0), Oi = R(0), Opr = R(0), Opi = R(0), Odr = R(0), Odi = R(0);
@@ -676,7 +682,7 @@ __device__ __forceinline__ void adjoint_cta(const MapParams<R>& P, const AdjPara
                         const R u1 = Opr * ba - Opi * bb;
                         const R u2 = Opr * bb + Opi * ba;
                         u3 = u1 * ba - u2 * bb;                 // Re(Omega_p z^2)
-                        const R ibp2 = R(1) / bp2;
+                        const R ibp2 = F::rcp_nr(bp2);
                         abar = nw * (GI * half_p1 * ba + R(2) * t1 + R(2) * q * ba * t3 * ibp2);
                         bbar = nw * (GI * half_p1 * bb - R(2) * t2 + R(2) * q * bb * t3 * ibp2);
                     }
@@ -757,7 +763,7 @@ __global__ void k_reduce_partials(const double* __restrict__ partial, long long 
                                   int n_theta, double* __restrict__ grad, double* __restrict__ chi2);
 
 template <int MODEL, int NF, int LPR, typename R>
-__global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<MODEL>())
+__global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<MODEL, R>())
 k_adjoint(const MapParams<R> P, const AdjParams<R> A, const R* __restrict__ gmaps,
           const R* __restrict__ target, R* __restrict__ maps_out, double* __restrict__ partial) {
     __shared__ AdjSmem<MODEL, NF, LPR, R> sm;
@@ -790,10 +796,15 @@ static int launch_adj_lpr(const MapParams<R>& P, const AdjParams<R>& A, const R*
 template <int MODEL, int NF, typename R>
 static int launch_adj_nf(const MapParams<R>& P, const AdjParams<R>& A, const R* gmaps, const R* target,
                          double* grad, double* chi2, R* maps, double* partial, cudaStream_t st) {
-    if (sizeof(R) == 8) return launch_adj_lpr<MODEL, NF, 32, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
-    const int lpr = lanes_per_ray(P.n_steps, P.n_pix);
-    if (lpr == 8) return launch_adj_lpr<MODEL, NF, 8, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
-    if (lpr == 16) return launch_adj_lpr<MODEL, NF, 16, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
+    if constexpr (sizeof(R) == 4) {
+        const int lpr = lanes_per_ray(P.n_steps, P.n_pix);
+        if (lpr == 8) return launch_adj_lpr<MODEL, NF, 8, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
+        if (lpr == 16) return launch_adj_lpr<MODEL, NF, 16, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
+    }
+    if constexpr (sizeof(R) == 8) {
+        if (lanes_per_ray_f64(P.n_pix) == 16)
+            return launch_adj_lpr<MODEL, NF, 16, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
+    }
     return launch_adj_lpr<MODEL, NF, 32, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
 }
 

@@ -37,15 +37,18 @@ namespace synax {
 // model's two-sample march also runs 5 (6 spill 64 bytes at 80 registers:
 // 0.260 against 0.251 ms for the Sec. 3.3 map at 16 lanes per ray).  The
 // other models keep 6 per SM (at most 85 registers), where they were measured.
+// FP64 runs 4 per SM (at most 128 registers; 3, or 168, with the grid model's
+// 8 cached FP64 nodes), where 1- and 2-frequency marches do not spill.
 // SYNAX_FWD_MIN_BLOCKS / SYNAX_FWD_THREADS override both at build time.
 #ifndef SYNAX_FWD_THREADS
 #define SYNAX_FWD_THREADS 128
 #endif
 constexpr int kThreads = SYNAX_FWD_THREADS;
-template <int MODEL> constexpr int fwd_min_blocks() {
+template <int MODEL, typename R> constexpr int fwd_min_blocks() {
 #ifdef SYNAX_FWD_MIN_BLOCKS
     return SYNAX_FWD_MIN_BLOCKS;
 #else
+    if (sizeof(R) == 8) return MODEL == SYNAX_MODEL_GRID ? 3 : 4;
     return MODEL == SYNAX_MODEL_JF12 || MODEL == SYNAX_MODEL_GRID ? 5 : 6;
 #endif
 }
@@ -55,7 +58,7 @@ template <int MODEL> constexpr int fwd_min_blocks() {
 // geometry, arm-tracker anchor, scan, rotation, reductions) over more samples
 // per lane; more lanes give more parallelism for few rays.
 template <int MODEL, int NF, int LPR, typename R>
-__global__ void __launch_bounds__(kThreads, fwd_min_blocks<MODEL>())
+__global__ void __launch_bounds__(kThreads, fwd_min_blocks<MODEL, R>())
 k_forward(const MapParams<R> P, R* __restrict__ maps) {
     using Ph = PhaseOps<R>;
     using PT = typename Ph::T;
@@ -144,10 +147,14 @@ static int launch_nf(const MapParams<R>& P, R* maps, cudaStream_t st) {
 
 template <int MODEL, int NF, typename R>
 static int launch_lpr(const MapParams<R>& P, R* maps, cudaStream_t st) {
-    if (sizeof(R) == 8) return launch_nf<MODEL, NF, 32, R>(P, maps, st);   // FP64: one width
-    const int lpr = lanes_per_ray(P.n_steps, P.n_pix);
-    if (lpr == 8) return launch_nf<MODEL, NF, 8, R>(P, maps, st);
-    if (lpr == 16) return launch_nf<MODEL, NF, 16, R>(P, maps, st);
+    if constexpr (sizeof(R) == 4) {
+        const int lpr = lanes_per_ray(P.n_steps, P.n_pix);
+        if (lpr == 8) return launch_nf<MODEL, NF, 8, R>(P, maps, st);
+        if (lpr == 16) return launch_nf<MODEL, NF, 16, R>(P, maps, st);
+    }
+    if constexpr (sizeof(R) == 8) {
+        if (lanes_per_ray_f64(P.n_pix) == 16) return launch_nf<MODEL, NF, 16, R>(P, maps, st);
+    }
     return launch_nf<MODEL, NF, 32, R>(P, maps, st);
 }
 

@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include "ffmath.cuh"
+#include "fx64.cuh"
 #include "status.cuh"
 #include "synax_internal.h"
 
@@ -165,33 +166,32 @@ template <> struct M<float> {
     }
 };
 
+// FP64: the fixed-point functions of fx64.cuh in place of CUDA's, which run on
+// the FP64 pipe (2 lanes per clock and SM) that bounds this march.
 template <> struct M<double> {
-    static __device__ __forceinline__ double exp(double x) { return ::exp(x); }
-    static __device__ __forceinline__ double log(double x) { return ::log(x); }
-    static __device__ __forceinline__ double div(double a, double b) { return a / b; }
-    static __device__ __forceinline__ double sqrt(double x) { return ::sqrt(x); }
+    static __device__ __forceinline__ double exp(double x) { return fx::exp_any<true>(x); }
+    static __device__ __forceinline__ double log(double x) { return fx::log_any<true>(x); }
+    static __device__ __forceinline__ double div(double a, double b) { return fx::div(a, b); }
+    static __device__ __forceinline__ double sqrt(double x) { return fx::sqrt(x); }
     static __device__ __forceinline__ double mulc(double x, double c) { return x * c; }
-    static __device__ __forceinline__ double rcp_nr(double x) { return 1.0 / x; }
-    static __device__ __forceinline__ double rsqrt_nr(double x) { return 1.0 / ::sqrt(x); }
+    static __device__ __forceinline__ double rcp_nr(double x) { return fx::rcp(x); }
     static __device__ __forceinline__ double mul_hl(double x, double hi, double lo) { return x * (hi + lo); }
-    static __device__ __forceinline__ double exp2_fast(double x) { return ::exp2(x); }
-    static __device__ __forceinline__ double exp_shape(double x) { return ::exp(x); }
-    static __device__ __forceinline__ double rcp_shape(double x) { return 1.0 / x; }
-    static __device__ __forceinline__ double rsqrt_shape(double x) { return 1.0 / ::sqrt(x); }
+    static __device__ __forceinline__ double exp2_fast(double x) { return fx::exp_any<false>(x); }
+    static __device__ __forceinline__ double exp_shape(double x) { return fx::exp_any<true>(x); }
+    static __device__ __forceinline__ double rcp_shape(double x) { return fx::rcp(x); }
+    static __device__ __forceinline__ double rsqrt_shape(double x) { return fx::rsqrt(x); }
     static __device__ __forceinline__ double mul_shape(double x, double c) { return x * c; }
-    static __device__ __forceinline__ double log2_fast(double x) { return ::log2(x); }
-    static __device__ __forceinline__ double rcp_fast(double x) { return 1.0 / x; }
-    static __device__ __forceinline__ double rsqrt_fast(double x) { return ::rsqrt(x); }
-    static __device__ __forceinline__ double atan2(double y, double x) { return ::atan2(y, x); }
+    static __device__ __forceinline__ double log2_fast(double x) { return fx::log_any<false>(x); }
+    static __device__ __forceinline__ double rcp_fast(double x) { return fx::rcp(x); }
+    static __device__ __forceinline__ double atan2(double y, double x) { return fx::atan2(y, x); }
     static __device__ __forceinline__ double floor(double x) { return ::floor(x); }
     static __device__ __forceinline__ double abs(double x) { return ::fabs(x); }
     static __device__ __forceinline__ double min(double a, double b) { return ::fmin(a, b); }
     static __device__ __forceinline__ double max(double a, double b) { return ::fmax(a, b); }
-    static __device__ __forceinline__ void sincos(double x, double* s, double* c) { ::sincos(x, s, c); }
-    static __device__ __forceinline__ void sincospi(double x, double* s, double* c) { ::sincospi(x, s, c); }
-    static __device__ __forceinline__ void sincos_rev(double r, double* s, double* c) {
-        ::sincospi(2.0 * r, s, c);
-    }
+    static __device__ __forceinline__ void sincos(double x, double* s, double* c) { fx::sincos_any<false>(x, s, c); }
+    static __device__ __forceinline__ void sincospi(double x, double* s, double* c) { fx::sincos_any<true>(0.5 * x, s, c); }
+    // sin and cos of 2 pi r
+    static __device__ __forceinline__ void sincos_rev(double r, double* s, double* c) { fx::sincos_any<true>(r, s, c); }
 };
 
 // ---------------------------------------------------------------------------
@@ -333,10 +333,8 @@ template <> struct PhaseOps<double> {
     static __device__ __forceinline__ T add(T a, T b) { return a + b; }
     static __device__ __forceinline__ T scale(T c, double d) { return c * d; }
     static __device__ __forceinline__ T scale2(T c, double d, double d_lo) { return c * (d + d_lo); }
-    static __device__ __forceinline__ double frac_mul(T c, T s) {
-        double x = c * s;
-        return x - rint(x);
-    }
+    // the whole product: sincos_rev drops the integer part exactly
+    static __device__ __forceinline__ double frac_mul(T c, T s) { return c * s; }
     static __device__ __forceinline__ T shfl_up(T v, int d, int width) {
         return __shfl_up_sync(0xffffffffu, v, d, width);
     }
@@ -416,28 +414,28 @@ __device__ __forceinline__ void healpix_los(int nside, long long pix, Los<R>& L)
     if (pix < ncap) {
         long long k = cap_ring(pix);
         long long j0 = pix - 2 * k * (k - 1);
-        R a = R(k * k) / R(3 * N * N);              // 1 - z
+        R a = M<R>::div(R(k * k), R(3 * N * N));              // 1 - z
         sinb = R(1) - a;
         cosb = M<R>::sqrt(a * (R(2) - a));
-        phi_pi = (R(j0) + R(0.5)) / R(2 * k);
+        phi_pi = M<R>::div((R(j0) + R(0.5)), R(2 * k));
     } else if (pix < npix - ncap) {
         long long pp = pix - ncap;
         long long i = N + pp / (4 * N);
         long long j0 = pp - (i - N) * 4 * N;
         long long s = (i - N + 1) & 1;
-        R z = R(4 * N - 2 * i) / R(3 * N);
+        R z = M<R>::div(R(4 * N - 2 * i), R(3 * N));
         sinb = z;
         cosb = M<R>::sqrt((R(1) - z) * (R(1) + z));
-        phi_pi = (R(j0) + (s ? R(0.5) : R(0))) / R(2 * N);
+        phi_pi = M<R>::div((R(j0) + (s ? R(0.5) : R(0))), R(2 * N));
     } else {
         long long c = npix - 1 - pix;
         long long k = cap_ring(c);
         long long m = c - 2 * k * (k - 1);
         long long j0 = 4 * k - 1 - m;
-        R a = R(k * k) / R(3 * N * N);
+        R a = M<R>::div(R(k * k), R(3 * N * N));
         sinb = a - R(1);
         cosb = M<R>::sqrt(a * (R(2) - a));
-        phi_pi = (R(j0) + R(0.5)) / R(2 * k);
+        phi_pi = M<R>::div((R(j0) + R(0.5)), R(2 * k));
     }
     R sl, cl;
     M<R>::sincospi(phi_pi, &sl, &cl);
@@ -507,8 +505,8 @@ __device__ __forceinline__ R box_exit(const R o[3], const R h[3], const R n[3]) 
     R t = R(1e30);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        if (n[k] > R(0)) t = M<R>::min(t, (h[k] - o[k]) / n[k]);
-        else if (n[k] < R(0)) t = M<R>::min(t, (-h[k] - o[k]) / n[k]);
+        if (n[k] > R(0)) t = M<R>::min(t, M<R>::div(h[k] - o[k], n[k]));
+        else if (n[k] < R(0)) t = M<R>::min(t, M<R>::div(-h[k] - o[k], n[k]));
     }
     return t;
 }
@@ -572,6 +570,43 @@ __device__ __forceinline__ R cr_density(R n0n, R rho, R az) {
     const R e2 = F::exp2_fast(R(-2.0 * kLog2e) * az);
     const R inv1 = F::rcp_fast(R(1) + e2);
     return n0n * F::exp2_fast(R(-0.2 * kLog2e) * rho) * (R(4) * e2 * inv1 * inv1);
+}
+// The same where sech^2 z is already known to FP64 accuracy (FP32 keeps its
+// own fast evaluation: the sech^2 of n_e is the accurate one).
+template <typename R>
+__device__ __forceinline__ R cr_density(R n0n, R rho, R az, R sech2) {
+    if constexpr (sizeof(R) == 8) return n0n * (fx::exp_radial<true>(rho) * sech2);
+    else return cr_density<R>(n0n, rho, az);
+}
+// sech^2 z and tanh |z| from e^{-2|z|}.
+template <typename R>
+__device__ __forceinline__ void sech2_tanh_of(R az, R& sech2, R& th) {
+    if constexpr (sizeof(R) == 8) {
+        fx::sech2_tanh(az, sech2, th);
+    } else {
+        const R e2 = M<R>::exp(R(-2) * az);
+        const R inv1 = M<R>::rcp_nr(R(1) + e2);
+        sech2 = R(4) * e2 * inv1 * inv1;
+        th = (R(1) - e2) * inv1;
+    }
+}
+// e^{-rho/20}, the radial profile of n_e.
+template <typename R>
+__device__ __forceinline__ R exp_rho20(R rho) {
+    if constexpr (sizeof(R) == 8) return fx::exp_radial<false>(rho);
+    else return M<R>::exp(-M<R>::mulc(rho, 0.05));
+}
+// 3 <= rho <= 20 (FP64: on the bits, without FP64 comparisons).
+template <typename R>
+__device__ __forceinline__ bool rho_in_range(R rho) {
+    if constexpr (sizeof(R) == 8) return !fx::above(3.0, rho) && !fx::above(rho, 20.0);
+    else return rho >= R(3) && rho <= R(20);
+}
+// B_perp^2 above the cut below which nothing is emitted.
+template <typename R>
+__device__ __forceinline__ bool is_lit(R bp2) {
+    if constexpr (sizeof(R) == 8) return fx::above(bp2, 1e-30);
+    else return bp2 > R(1e-30);
 }
 
 // Position in the JF12 spiral-arm pattern: sector k in 0..7 and fraction
@@ -768,6 +803,7 @@ struct FieldLocal {
     R gfx, gfy, gfz;     // fractional position in the cell
     // stacked WMAP: cos/sin of each component's psi and chi
     R kcp[4], ksp[4], kcc[4], ksc[4];
+    R gw[8];                  // grid model, FP64: the trilinear weights of the sample
     // input set by the FP32 marches before eval: on a ray of constant z (the
     // HEALPix equator ring, n_z = 0) the vertical n_e profile sech^2 z is the
     // same at every sample, so its FP32 rounding would be a coherent relative
@@ -834,16 +870,14 @@ template <> struct Model<SYNAX_MODEL_WMAP> {
         const R c = has_rho ? x * ri : R(1);
         const R s = has_rho ? y * ri : R(0);
         const R az = F::abs(z);
-        const R e2 = F::exp(R(-2) * az);                      // e^{-2|z|}
-        const R inv1 = F::rcp_nr(R(1) + e2);
-        const R sech2 = R(4) * e2 * inv1 * inv1;
+        R sech2, thz;                                         // sech^2 z, tanh |z|
+        sech2_tanh_of(az, sech2, thz);
         R psi = R(0), chi = R(0), lnr8 = R(0), th = R(0);
-        const bool in_range = rho >= R(3) && rho <= R(20);
+        const bool in_range = rho_in_range(rho);
         if (in_range) {
             lnr8 = F::log(rho * R(0.125));
             psi = m[mc::W_PSI0] + m[mc::W_PSI1] * lnr8;
-            th = (R(1) - e2) * inv1;                         // tanh |z|
-            th = z < R(0) ? -th : th;
+            th = z < R(0) ? -thz : thz;
             chi = m[mc::W_CHI0] * th;
         }
         const R env = F::exp(-(F::mulc(rho, 0.125) + az));
@@ -855,9 +889,9 @@ template <> struct Model<SYNAX_MODEL_WMAP> {
         B[0] = br * c - bp * s + m[mc::W_BUX];
         B[1] = br * s + bp * c;
         B[2] = amp * sc;
-        const R n0u = cr_density<R>(m[mc::W_N0U], rho, az);
+        const R n0u = cr_density<R>(m[mc::W_N0U], rho, az, sech2);
         N0 = m[mc::W_N0OBS] * n0u;
-        const R er = F::exp(-F::mulc(rho, 0.05));
+        const R er = exp_rho20(rho);
         const R neu = loc.flat_z ? F::mul_hl(er, loc.zc_hi, loc.zc_lo) : er * sech2;
         ne = F::mul_hl(neu, m[mc::W_NE0], m[mc::W_NE0_LO]);
         loc.c = c; loc.s = s; loc.az = az; loc.rho = rho;
@@ -976,11 +1010,10 @@ template <> struct Model<SYNAX_MODEL_WMAP_STACK> {
         const R c = has_rho ? x * ri : R(1);
         const R s = has_rho ? y * ri : R(0);
         const R az = F::abs(z);
-        const R e2 = F::exp(R(-2) * az);                      // e^{-2|z|}
-        const R inv1 = F::rcp_nr(R(1) + e2);
-        const bool in_range = rho >= R(3) && rho <= R(20);
+        R sech2, th;                                          // sech^2 z, tanh |z|
+        sech2_tanh_of(az, sech2, th);
+        const bool in_range = rho_in_range(rho);
         const R lnr8 = in_range ? F::log(rho * R(0.125)) : R(0);
-        R th = (R(1) - e2) * inv1;                             // tanh |z|
         th = z < R(0) ? -th : th;
         // unit vector of each component, scaled by its weight times b0 (a
         // host product kept as hi + lo: the rounding of these magnitudes would
@@ -1010,10 +1043,10 @@ template <> struct Model<SYNAX_MODEL_WMAP_STACK> {
         B[0] = comp[0][0] + comp[1][0] + comp[2][2] + comp[3][1];
         B[1] = comp[0][1] + comp[1][2] + comp[2][1] + comp[3][0];
         B[2] = comp[0][2] + comp[1][1] + comp[2][0] + comp[3][2];
-        const R n0u = cr_density<R>(m[mc::S_N0U], rho, az);
+        const R n0u = cr_density<R>(m[mc::S_N0U], rho, az, sech2);
         N0 = m[mc::S_N0OBS] * n0u;
-        const R er = F::exp(-F::mulc(rho, 0.05));
-        const R neu = loc.flat_z ? F::mul_hl(er, loc.zc_hi, loc.zc_lo) : er * (R(4) * e2 * inv1 * inv1);
+        const R er = exp_rho20(rho);
+        const R neu = loc.flat_z ? F::mul_hl(er, loc.zc_hi, loc.zc_lo) : er * sech2;
         ne = F::mul_hl(neu, m[mc::S_NE0], m[mc::S_NE0_LO]);
         loc.c = c; loc.s = s; loc.lnr8 = lnr8; loc.thz = th; loc.in_range = in_range ? R(1) : R(0);
         loc.n0_unit = n0u; loc.ne_unit = neu;
@@ -1054,6 +1087,14 @@ __device__ __forceinline__ int grid_axis_split(R cf, R f, R umax, R& fout) {
     return (int)M<R>::min(M<R>::max(cf, R(0)), umax - R(1));
 }
 
+// The same from an integer whole part (FP64: no FP64 comparison or conversion).
+__device__ __forceinline__ int grid_axis_split_int(long long ci, double f, int n, double& fout) {
+    const int last = n - 2;
+    f = ci < 0 ? 0.0 : f;
+    fout = ci > last ? 1.0 : f;
+    return ci < 0 ? 0 : (ci > last ? last : (int)ci);
+}
+
 // Direct form for an arbitrary point: u = x (n - 1)/l + (n - 1)/2.
 template <typename R>
 __device__ __forceinline__ int grid_axis(R x, R s, R slo, R o, R umax, R& f) {
@@ -1084,6 +1125,7 @@ template <typename R>
 struct GridRay {
     R ia[3], a[3], du[3], dulo[3];
     int na;
+    int ii[3];                // FP64: ia as integers
 };
 
 template <typename R>
@@ -1113,6 +1155,7 @@ __device__ __forceinline__ void grid_ray_init(const MapParams<R>& P, const Los<R
             const R fl = M<R>::floor(u);
             g.ia[k] = fl;
             g.a[k] = u - fl;
+            g.ii[k] = (int)M<R>::min(M<R>::max(fl, R(-1073741824)), R(1073741824));
             g.du[k] = P.m[mc::G_S + k] * L.n[k] * dr;
             g.dulo[k] = R(0);
         }
@@ -1120,20 +1163,33 @@ __device__ __forceinline__ void grid_ray_init(const MapParams<R>& P, const Los<R
 }
 
 template <typename R>
-__device__ __forceinline__ int grid_locate_ray(const MapParams<R>& P, const GridRay<R>& g, int n, R& fx, R& fy,
-                                               R& fz) {
-    const R kf = R(n - g.na);
+__device__ __forceinline__ int grid_locate_ray(const MapParams<R>& P, const GridRay<R>& g, int n, R& fx_, R& fy_,
+                                               R& fz_) {
     R fr[3];
     int c[3];
+    if constexpr (sizeof(R) == 8) {
+        const R kd = fx::from_int(n - g.na);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            int whole;
+            const R f = fx::split_floor(fma(kd, g.du[k], g.a[k]), whole);
+            c[k] = grid_axis_split_int((long long)g.ii[k] + whole, f, P.grid_n[k], fr[k]);
+        }
+        fx_ = fr[0];
+        fy_ = fr[1];
+        fz_ = fr[2];
+        return (c[2] * P.grid_n[1] + c[1]) * P.grid_n[0] + c[0];
+    }
+    const R kf = R(n - g.na);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const R v = fma(kf, g.du[k], fma(kf, g.dulo[k], g.a[k]));
         const R fl = M<R>::floor(v);
         c[k] = grid_axis_split<R>(g.ia[k] + fl, v - fl, P.m[mc::G_UMAX + k], fr[k]);
     }
-    fx = fr[0];
-    fy = fr[1];
-    fz = fr[2];
+    fx_ = fr[0];
+    fy_ = fr[1];
+    fz_ = fr[2];
     return (c[2] * P.grid_n[1] + c[1]) * P.grid_n[0] + c[0];
 }
 
@@ -1161,6 +1217,18 @@ __device__ __forceinline__ void grid_load(const MapParams<R>& P, int base, GridC
         const R v010 = __ldg(p + sy + c), v110 = __ldg(p + sy + 3 + c);
         const R v001 = __ldg(p + sz + c), v101 = __ldg(p + sz + 3 + c);
         const R v011 = __ldg(p + sz + sy + c), v111 = __ldg(p + sz + sy + 3 + c);
+        if constexpr (sizeof(R) == 8) {
+            // the nodes themselves: the differences would be 14 FP64 additions per component and cell
+            gc.a[c] = v000;
+            gc.b[c] = v100;
+            gc.c[c] = v010;
+            gc.d[c] = v110;
+            gc.e[c] = v001;
+            gc.f[c] = v101;
+            gc.g[c] = v011;
+            gc.h[c] = v111;
+            continue;
+        }
         const R bx0 = v100 - v000, bx1 = v110 - v010, bx2 = v101 - v001, bx3 = v111 - v011;
         gc.a[c] = v000;
         gc.b[c] = bx0;
@@ -1174,7 +1242,16 @@ __device__ __forceinline__ void grid_load(const MapParams<R>& P, int base, GridC
     gc.base = base;
 }
 
-// Trilinear blend at (fx, fy, fz) of the cached cell.
+// The blend of the cached nodes with the 8 trilinear weights (FP64).
+__device__ __forceinline__ void grid_blend_nodes(const GridCell<double>& gc, const double w[8], double B[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double lo = fma(w[3], gc.d[c], fma(w[2], gc.c[c], fma(w[1], gc.b[c], w[0] * gc.a[c])));
+        B[c] = fma(w[7], gc.h[c], fma(w[6], gc.g[c], fma(w[5], gc.f[c], fma(w[4], gc.e[c], lo))));
+    }
+}
+
+// Trilinear blend at (fx, fy, fz) of the cached cell (FP32: its coefficients).
 template <typename R>
 __device__ __forceinline__ void grid_blend(const GridCell<R>& gc, R fx, R fy, R fz, R B[3]) {
 #pragma unroll
@@ -1188,26 +1265,31 @@ __device__ __forceinline__ void grid_blend(const GridCell<R>& gc, R fx, R fy, R 
 // Fields of the grid model at a sample in cell `base` with fractions
 // (fx, fy, fz) and position (x, y, z) (for N0 and n_e).
 template <typename R>
-__device__ __forceinline__ void grid_eval(const MapParams<R>& P, GridCell<R>& gc, int base, R fx, R fy, R fz,
+__device__ __forceinline__ void grid_eval(const MapParams<R>& P, GridCell<R>& gc, int base, R fx_, R fy_, R fz_,
                                           R x, R y, R z, R B[3], R& N0, R& ne, FieldLocal<R>& loc) {
     using F = M<R>;
     if (base != gc.base) grid_load<R>(P, base, gc);
-    grid_blend<R>(gc, fx, fy, fz, B);
+    if constexpr (sizeof(R) == 8) {
+        fx::trilinear_weights(fx_, fy_, fz_, loc.gw);
+        grid_blend_nodes(gc, loc.gw, B);
+    } else {
+        grid_blend<R>(gc, fx_, fy_, fz_, B);
+    }
     const R rho = F::sqrt(x * x + y * y);
     const R az = F::abs(z);
-    const R e2 = F::exp(R(-2) * az);                          // e^{-2|z|}
-    const R inv1 = F::rcp_nr(R(1) + e2);
-    const R n0u = cr_density<R>(P.m[mc::G_N0U], rho, az);
+    R sech2, th;
+    sech2_tanh_of(az, sech2, th);
+    const R n0u = cr_density<R>(P.m[mc::G_N0U], rho, az, sech2);
     N0 = P.m[mc::G_N0OBS] * n0u;
-    const R er = F::exp(-F::mulc(rho, 0.05));
-    const R neu = loc.flat_z ? F::mul_hl(er, loc.zc_hi, loc.zc_lo) : er * (R(4) * e2 * inv1 * inv1);
+    const R er = exp_rho20(rho);
+    const R neu = loc.flat_z ? F::mul_hl(er, loc.zc_hi, loc.zc_lo) : er * sech2;
     ne = F::mul_hl(neu, P.m[mc::G_NE0], P.m[mc::G_NE0_LO]);
     loc.n0_unit = n0u;
     loc.ne_unit = neu;
     loc.gbase = base;
-    loc.gfx = fx;
-    loc.gfy = fy;
-    loc.gfz = fz;
+    loc.gfx = fx_;
+    loc.gfy = fy_;
+    loc.gfz = fz_;
 }
 
 // ---------------------------------------------------------------------------
@@ -1245,10 +1327,11 @@ __device__ __forceinline__ Emit<R> emit(const R B[3], R N0, R ne, const Los<R>& 
     R bn, bb;
     dot_n_eb<R>(B, L, bn, bb);
     const R bl = B[0] * L.el[0] + B[1] * L.el[1];
-    const R bp2 = bl * bl + bb * bb;
+    const R bl2 = bl * bl, bb2 = bb * bb;
+    const R bp2 = sizeof(R) == 8 ? bl2 + bb2 : bl * bl + bb * bb;
     // B_perp below 1e-15 uG radiates nothing measurable; the cut also keeps
     // FP32 denormals away from the flush-to-zero logarithm.
-    const R w = bp2 > R(1e-30) ? M<R>::exp2_fast(q * M<R>::log2_fast(bp2)) : R(0);
+    const R w = is_lit<R>(bp2) ? M<R>::exp2_fast(q * M<R>::log2_fast(bp2)) : R(0);
     const R nw = N0 * w;
     Emit<R> e;
     e.jI = nw * bp2;
@@ -1257,8 +1340,8 @@ __device__ __forceinline__ Emit<R> emit(const R B[3], R N0, R ne, const Los<R>& 
         e.pc = v.x;
         e.ps = v.y;
     } else {
-        e.pc = nw * (bl * bl - bb * bb);
-        e.ps = nw * (R(2) * bl * bb);
+        e.pc = nw * (bl2 - bb2);
+        e.ps = (nw + nw) * (bl * bb);
     }
     e.f = -ne * bn;
     return e;
@@ -1809,9 +1892,9 @@ __device__ __forceinline__ void march_lane(const MapParams<R>& P, const R* s_arm
     R nh = R(n0) + R(0.5);                              // n + 1/2, exact
     FlatZ fzr{false, 0.0f, 0.0f};
     if constexpr (sizeof(R) == 4) fzr = flat_z_of(P, nd);
-#pragma unroll 2
+#pragma unroll (sizeof(R) == 8 ? 1 : 2)
     for (int n = n0; n < n1; ++n, nh += R(1)) {
-        const R t = fma(nh, dr, nh * dr_lo);            // (n + 1/2) dr, dr as hi + lo
+        const R t = sizeof(R) == 8 ? nh * dr : fma(nh, dr, nh * dr_lo);   // (n + 1/2) dr, dr as hi + lo (FP64: lo is 0)
         R x, y, z;
         sample_pos<MODEL, R>(P, L, nd, t, x, y, z);
         R B[3], N0, ne;
@@ -1837,7 +1920,7 @@ __device__ __forceinline__ void march_lane(const MapParams<R>& P, const R* s_arm
         if constexpr (sizeof(R) == 4) {
             ff_add_f_pair(S, make_float2(P.w_own * e.f, e.f), s_n, S);
         } else {
-            s_n = Ph::add(S, P.w_own * e.f);
+            s_n = fma(P.w_own, e.f, S);
             S = Ph::add(S, e.f);
         }
         if constexpr (sizeof(R) == 4 && NF >= 2) {
@@ -1860,8 +1943,8 @@ __device__ __forceinline__ void march_lane(const MapParams<R>& P, const R* s_arm
                 if (k < P.n_freq) {
                     R sn, cs;
                     M<R>::sincos_rev(Ph::frac_mul(cd[k], s_n), &sn, &cs);
-                    zr[k] += e.pc * cs - e.ps * sn;         // (pc + i ps) e^{i phi}
-                    zi[k] += e.pc * sn + e.ps * cs;
+                    zr[k] = fma(e.pc, cs, fma(-e.ps, sn, zr[k]));   // (pc + i ps) e^{i phi}
+                    zi[k] = fma(e.pc, sn, fma(e.ps, cs, zi[k]));
                 }
             }
         }
@@ -1899,7 +1982,7 @@ __device__ __forceinline__ void ray_setup(const MapParams<R>& P, long long ray, 
         }
     } else {
         healpix_los<R>(P.nside, P.pix_begin + ray, L);
-        dr = P.box_clip ? box_exit<R>(P.obs, P.box_half, L.n) / R(P.n_steps) : P.dr;
+        dr = P.box_clip ? M<R>::div(box_exit<R>(P.obs, P.box_half, L.n), R(P.n_steps)) : P.dr;
         dr_lo = P.box_clip ? R(0) : P.dr_lo;
     }
 }

@@ -107,6 +107,7 @@ double observer_n0_norm(const synax_problem& P);
 // Lanes per ray (32, 16 or 8) for a map of n_pix rays of n_steps samples:
 // the launch tuning table (tune.cu), overridable per process.
 int lanes_per_ray(int n_steps, long long n_pix);
+int lanes_per_ray_f64(long long n_pix);
 
 // Host-side entry points into the kernels (forward.cu, adjoint.cu).
 int launch_forward_f32(const MapParams<float>& P, void* maps, void* stream);

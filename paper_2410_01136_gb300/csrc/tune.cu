@@ -4,7 +4,7 @@
 // fill the GPU several times over; otherwise keep 32 lanes per ray for
 // parallelism.  synax_set_lanes_per_ray() installs a measured table (the
 // autotuner in paper_2410_01136_gb300/tune.py times the candidates and
-// writes it) or forces one value.
+// writes it) or forces one value.  FP64 has a rule of its own.
 #include <atomic>
 
 #include "synax_internal.h"
@@ -36,6 +36,15 @@ int lanes_per_ray(int n_steps, long long n_pix) {
     if (n_steps >= 64 && n_pix >= rays_needed_8 / 2) return 16;
     return 32;
 }
+
+// FP64: the per-lane set-up and reductions weigh more than in FP32 (their FP64
+// instructions run at 2 lanes per clock and SM), so 16 lanes per ray as soon as
+// that gives every SM a CTA of 128 threads.  Measured at 32, 16 and 8 lanes:
+// grid map of Nside 64, 512 steps 4.18, 4.03, 4.02 ms; JF12-type map of
+// Nside 64, 200 steps 4.35, 3.94, 3.83 ms; WMAP-type map of Nside 16, 128
+// steps 0.122, 0.106, 0.169 ms; JF12-type map + gradient of Nside 16, 100
+// steps 0.902, 0.783, 1.027 ms.
+int lanes_per_ray_f64(long long n_pix) { return n_pix >= 8LL * 152 ? 16 : 32; }
 
 }  // namespace synax
 
