@@ -185,7 +185,15 @@ __device__ __forceinline__ void epilogue16(const GemmEpiParams& ep, const float*
         float z16[16], b[16], a[16], t[16];
         if constexpr (EPI == EPI_BIAS_GELU || EPI == EPI_MSE) load16(ep.bias, col0, nv, b);
         if constexpr (EPI == EPI_GELU_BWD) load16(ep.aux + (long long)row * ep.ld_aux, col0, nv, a);
-        if constexpr (EPI == EPI_MSE) load16(ep.target + trow * ep.ld_target, col0, nv, t);
+        if constexpr (EPI == EPI_MSE) {
+            load16(ep.target + trow * ep.ld_target, col0, nv, t);
+            if (ep.target_mean) {
+                float mu[16];
+                load16(ep.target_mean, col0, nv, mu);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) t[i] = __fmul_rn(t[i] - mu[i], ep.target_scale);
+            }
+        }
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             float x = v[i];

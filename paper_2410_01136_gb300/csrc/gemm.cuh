@@ -44,6 +44,8 @@ struct GemmEpiParams {
     const float* target;         // EPI_MSE: target rows, [*][ld_target]
     int ld_target;
     const int* target_rows;      // EPI_MSE: row m reads target row target_rows[m]
+    const float* target_mean;    // EPI_MSE: the target is (target - target_mean[n]) * target_scale (null: as it is)
+    float target_scale;
     float coef;                  // EPI_MSE: gradient factor 2 / (rows * cols)
     float* loss_partial;         // EPI_MSE: one float per CTA (gemm_tiles of them)
     float scale;                 // EPI_AFFINE, EPI_SCALE_ACC

@@ -24,9 +24,9 @@
 // from the FP32 master weights after every update.
 //
 // Training.  One step = gather a batch (counter-based Feistel shuffle of the
-// stored samples per epoch), forward, MSE, backward, bias gradients, Adam
-// (cosine learning-rate schedule), loss bookkeeping -- 21 kernels for 4
-// hidden layers, captured once into a CUDA graph and replayed; the step
+// stored samples per epoch), forward, MSE, backward, then bias gradients, Adam
+// (cosine learning-rate schedule) and loss bookkeeping in one kernel -- 16
+// kernels for 4 hidden layers, captured once into a CUDA graph and replayed; the step
 // counter lives in device memory so replays advance it.  Everything is
 // deterministic (no atomics in any sum), so a restored checkpoint replays
 // the same loss curve bit for bit.
@@ -44,6 +44,7 @@
 #include <new>
 #include <vector>
 
+#include "fx64.cuh"
 #include "gemm.cuh"
 #include "srht.cuh"
 #include "synax_internal.h"
@@ -136,6 +137,26 @@ __device__ uint32_t feistel_perm(uint32_t i, uint32_t n, int half_bits, uint64_t
     return i;   // not reached: the cycle of i re-enters [0, n)
 }
 
+struct AdamHyper {
+    float lr0, lr_min, beta1, beta2, eps;
+    int total_steps;
+    double ln_beta1, ln_beta2;
+};
+
+// Step size and bias corrections of the coming step t + 1, into coef[0..2] =
+// (lr, 1 - beta1^(t+1), 1 - beta2^(t+1)): one thread of the step's first
+// kernel, with the powers as exponentials of fx64.cuh (a kernel of its own
+// with CUDA's FP64 pow and cos took 11 us of every step).
+__device__ inline void adam_prep(const AdamHyper& h, int t, float* coef) {
+    const int t1 = t + 1;
+    const double s = (double)min(t, h.total_steps) / (double)max(h.total_steps, 1);
+    double sn, cs;
+    fx::sincos_any<true>(0.5 * s, &sn, &cs);
+    coef[0] = (float)(h.lr_min + 0.5 * ((double)h.lr0 - h.lr_min) * (1.0 + cs));
+    coef[1] = (float)(1.0 - fx::exp_any<true>((double)t1 * h.ln_beta1));
+    coef[2] = (float)(1.0 - fx::exp_any<true>((double)t1 * h.ln_beta2));
+}
+
 struct GatherArgs {
     const float* theta;     // [*][ld] physical parameters
     int ld;
@@ -152,6 +173,9 @@ struct GatherArgs {
     uint32_t steps_per_epoch;
     uint64_t seed;
     const int* t_dev;
+    // Adam's coefficients of the coming step (null: not a training step)
+    float* coef;
+    AdamHyper hyper;
 };
 
 // One warp per batch row: lane 0 finds the source sample, the lanes write
@@ -160,6 +184,7 @@ __global__ void k_gather_input(GatherArgs a) {
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     tc::launch_dependents();
+    if (a.coef && b == 0 && lane == 31) adam_prep(a.hyper, *a.t_dev, a.coef);
     if (b >= a.B) return;
     uint32_t src = (uint32_t)b;
     if (a.n) {
@@ -238,37 +263,6 @@ struct LayerTable {
     const bf16* dZt[kMaxLayers];  // [N_l][B]
 };
 
-// db[boff_l + j] = sum_b dZ_l[b][j], one warp per output row, fixed order.
-__global__ void k_bias_grad(LayerTable T, int B, float* __restrict__ db) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    int l = 0, j = warp;
-    while (l < T.L && j >= T.rows[l]) j -= T.rows[l++];
-    if (l >= T.L) return;
-    const bf16* src = T.dZt[l] + (long long)j * B;
-    float s = 0.0f;
-    for (int b = lane; b < B; b += 32) s += __bfloat162float(src[b]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) db[T.boff[l] + j] = s;
-}
-
-struct AdamHyper {
-    float lr0, lr_min, beta1, beta2, eps;
-    int total_steps;
-};
-
-// Step size and bias corrections of the coming step t + 1, computed once per
-// step (one thread) into coef[0..2] = (lr, 1 - beta1^(t+1), 1 - beta2^(t+1)).
-__global__ void k_adam_prep(AdamHyper h, const int* t_dev, float* coef) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int t1 = *t_dev + 1;
-    const double s = (double)min(t1 - 1, h.total_steps) / (double)max(h.total_steps, 1);
-    coef[0] = (float)(h.lr_min + 0.5 * ((double)h.lr0 - h.lr_min) * (1.0 + cos(3.14159265358979323846 * s)));
-    coef[1] = (float)(1.0 - pow((double)h.beta1, (double)t1));
-    coef[2] = (float)(1.0 - pow((double)h.beta2, (double)t1));
-}
-
 __device__ inline float adam_update(float w, float g, float& m, float& v, const AdamHyper& h, float lr, float bc1,
                                     float bc2) {
     m = h.beta1 * m + (1.0f - h.beta1) * g;
@@ -276,75 +270,140 @@ __device__ inline float adam_update(float w, float g, float& m, float& v, const 
     return w - lr * (m / bc1) / (sqrtf(v / bc2) + h.eps);
 }
 
-// Adam on the weights (update != 0) and the BF16 copies W and W^T, in 32x32
-// tiles so that the transposed copy is written coalesced.
-__global__ void __launch_bounds__(256)
-k_adam_weights(LayerTable T, float* __restrict__ W, const float* __restrict__ G, float* __restrict__ Mw,
-               float* __restrict__ Vw, bf16* __restrict__ Wb, bf16* __restrict__ Wt, AdamHyper h,
-               const float* __restrict__ coef, int update) {
-    __shared__ bf16 tile[32][34];
+// One 64 x 64 tile of a layer's weights: Adam (update) and the BF16 copies W
+// and W^T.  Rows and columns of every layer are multiples of 64.  HBM-bound:
+// 32 B per parameter (w, m, v read and written, g read, 2 BF16 copies).  A
+// thread keeps 16 16-byte loads in flight (4 rows of w, g, m, v); the
+// transposed copy goes through shared memory so that both copies are written
+// in runs of 128 bytes.  12.6 M parameters from a cold L2: 78 us with 32 x 32
+// tiles of 4-byte accesses; 72 us so, biases and loss included (403 MB at 5.6 TB/s).
+__device__ __forceinline__ void adam_tile(const LayerTable& T, int block, float* __restrict__ W,
+                                          const float* __restrict__ G, float* __restrict__ Mw,
+                                          float* __restrict__ Vw, bf16* __restrict__ Wb, bf16* __restrict__ Wt,
+                                          const AdamHyper& h, const float* __restrict__ coef, int update) {
+    __shared__ uint32_t tile[64][33];       // 2 BF16 of a row each; the 33rd keeps every fourth row 4 banks apart
     int l = 0;
-    while (l + 1 < T.L && (int)blockIdx.x >= T.tile_begin[l + 1]) ++l;
+    while (l + 1 < T.L && block >= T.tile_begin[l + 1]) ++l;
     const int rows = T.rows[l], cols = T.cols[l];
-    const int local = blockIdx.x - T.tile_begin[l];
-    const int tiles_c = (cols + 31) / 32;
-    const int tr = local / tiles_c, tc = local % tiles_c;
-    float lr = 0.f, bc1 = 1.f, bc2 = 1.f;
-    if (update) {
-        lr = coef[0];
-        bc1 = coef[1];
-        bc2 = coef[2];
-    }
+    const int local = block - T.tile_begin[l];
+    const int tiles_c = cols / 64;
+    const int r0 = (local / tiles_c) * 64, c0 = (local % tiles_c) * 64;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const long long off = T.woff[l];
+    long long i[4];
+    float4 w[4], g[4], m[4], v[4];
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int r = tr * 32 + threadIdx.y + 8 * k, c = tc * 32 + threadIdx.x;
-        if (r < rows && c < cols) {
-            const long long i = off + (long long)r * cols + c;
-            float w = W[i];
-            if (update) {
-                float m = Mw[i], v = Vw[i];
-                w = adam_update(w, G[i], m, v, h, lr, bc1, bc2);
-                W[i] = w;
-                Mw[i] = m;
-                Vw[i] = v;
-            }
-            const bf16 wb = __float2bfloat16_rn(w);
-            Wb[i] = wb;
-            tile[threadIdx.y + 8 * k][threadIdx.x] = wb;
+        i[k] = off + (long long)(r0 + ty + 16 * k) * cols + c0 + 4 * tx;
+        w[k] = *reinterpret_cast<const float4*>(W + i[k]);
+        if (update) {
+            g[k] = *reinterpret_cast<const float4*>(G + i[k]);
+            m[k] = *reinterpret_cast<const float4*>(Mw + i[k]);
+            v[k] = *reinterpret_cast<const float4*>(Vw + i[k]);
         }
     }
-    __syncthreads();
+    if (update) {
+        const float lr = coef[0], bc1 = coef[1], bc2 = coef[2];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            w[k].x = adam_update(w[k].x, g[k].x, m[k].x, v[k].x, h, lr, bc1, bc2);
+            w[k].y = adam_update(w[k].y, g[k].y, m[k].y, v[k].y, h, lr, bc1, bc2);
+            w[k].z = adam_update(w[k].z, g[k].z, m[k].z, v[k].z, h, lr, bc1, bc2);
+            w[k].w = adam_update(w[k].w, g[k].w, m[k].w, v[k].w, h, lr, bc1, bc2);
+            *reinterpret_cast<float4*>(W + i[k]) = w[k];
+            *reinterpret_cast<float4*>(Mw + i[k]) = m[k];
+            *reinterpret_cast<float4*>(Vw + i[k]) = v[k];
+        }
+    }
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int c = tc * 32 + threadIdx.y + 8 * k, r = tr * 32 + threadIdx.x;
-        if (r < rows && c < cols) Wt[off + (long long)c * rows + r] = tile[threadIdx.x][threadIdx.y + 8 * k];
+        const uint2 p = make_uint2(pack_bf16x2(w[k].x, w[k].y), pack_bf16x2(w[k].z, w[k].w));
+        *reinterpret_cast<uint2*>(Wb + i[k]) = p;
+        tile[ty + 16 * k][2 * tx] = p.x;
+        tile[ty + 16 * k][2 * tx + 1] = p.y;
+    }
+    __syncthreads();
+    // W^T: this thread's 4 rows (4 tx ..) of column ty + 16 k
+    const unsigned short* ts = reinterpret_cast<const unsigned short*>(tile);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int c = ty + 16 * k;
+        const uint32_t e0 = ts[(4 * tx + 0) * 66 + c], e1 = ts[(4 * tx + 1) * 66 + c];
+        const uint32_t e2 = ts[(4 * tx + 2) * 66 + c], e3 = ts[(4 * tx + 3) * 66 + c];
+        *reinterpret_cast<uint2*>(Wt + off + (long long)(c0 + c) * rows + r0 + 4 * tx) =
+            make_uint2(e0 | (e1 << 16), e2 | (e3 << 16));
     }
 }
 
-__global__ void k_adam_bias(float* __restrict__ b, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int n, AdamHyper h, const float* __restrict__ coef) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float lr = coef[0], bc1 = coef[1], bc2 = coef[2];
-    float mi = m[i], vi = v[i];
-    b[i] = adam_update(b[i], g[i], mi, vi, h, lr, bc1, bc2);
-    m[i] = mi;
-    v[i] = vi;
+// The BF16 copies alone (new weights).
+__global__ void __launch_bounds__(256) k_refresh_copies(LayerTable T, float* W, bf16* Wb, bf16* Wt) {
+    adam_tile(T, blockIdx.x, W, nullptr, nullptr, nullptr, Wb, Wt, AdamHyper{}, nullptr, 0);
 }
 
-// loss = sum of the CTA partials (fixed order) / count; advance the step.
-__global__ void k_finalize(const float* __restrict__ part, int n_part, float inv_count, float* __restrict__ hist,
-                           int* t_dev, int update, float* loss_out) {
-    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
-    double s = 0.0;
-    for (int i = threadIdx.x; i < n_part; i += 32) s += part[i];
+struct UpdateArgs {
+    LayerTable T;
+    int B;
+    float *W, *dW, *mW, *vW;
+    bf16 *Wb, *Wt;
+    float *b, *db, *mb, *vb;
+    int bias_blocks;              // 8 biases each
+    AdamHyper h;
+    const float* coef;
+    int update;
+    const float* loss_part;
+    int n_part;
+    float inv_count;
+    float *loss_hist, *loss_out;
+    int* t_dev;
+};
+
+// The end of a step in one launch, whose parts do not depend on one another:
+//   block 0: loss = sum of the CTA partials (fixed order) / count, step counter;
+//   bias_blocks: db[boff_l + j] = sum_b dZ_l[b][j], one warp per bias in fixed
+//     order, and (update) Adam on that bias;
+//   the rest (update): Adam on the weights, one tile per block.
+// As four kernels (7 + 3 + 4 us beside the weights' 78) they ran one after another.
+__global__ void __launch_bounds__(256, 2) k_update(const __grid_constant__ UpdateArgs a) {
+    tc::grid_dependency_wait();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int block = blockIdx.x;
+    if (block == 0) {
+        if (warp != 0) return;
+        double s = 0.0;
+        for (int i = lane; i < a.n_part; i += 32) s += a.loss_part[i];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x != 0) return;
-    const float loss = (float)(s * inv_count);
-    const int t = *t_dev;
-    hist[t & (kLossHist - 1)] = loss;
-    if (loss_out) *loss_out = loss;
-    if (update) *t_dev = t + 1;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane != 0) return;
+        const float loss = (float)(s * a.inv_count);
+        const int t = *a.t_dev;
+        a.loss_hist[t & (kLossHist - 1)] = loss;
+        if (a.loss_out) *a.loss_out = loss;
+        if (a.update) *a.t_dev = t + 1;
+        return;
+    }
+    block -= 1;
+    if (block < a.bias_blocks) {
+        int l = 0, j = block * 8 + warp;
+        while (l < a.T.L && j >= a.T.rows[l]) j -= a.T.rows[l++];
+        if (l >= a.T.L) return;
+        const bf16* src = a.T.dZt[l] + (long long)j * a.B;
+        float s = 0.0f;
+#pragma unroll 8
+        for (int b = lane; b < a.B; b += 32) s += __bfloat162float(src[b]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane != 0) return;
+        const int i = a.T.boff[l] + j;
+        a.db[i] = s;
+        if (a.update) {
+            float mi = a.mb[i], vi = a.vb[i];
+            a.b[i] = adam_update(a.b[i], s, mi, vi, a.h, a.coef[0], a.coef[1], a.coef[2]);
+            a.mb[i] = mi;
+            a.vb[i] = vi;
+        }
+        return;
+    }
+    adam_tile(a.T, block - a.bias_blocks, a.W, a.dW, a.mW, a.vW, a.Wb, a.Wt, a.h, a.coef, 1);
 }
 
 // Per-column mean and mean squared deviation of y [n][n_out] (two passes,
@@ -483,7 +542,6 @@ struct synax_surrogate_s {
     float* Z[kMaxLayers] = {nullptr};
     bf16 *dZ[kMaxLayers] = {nullptr}, *dZt[kMaxLayers] = {nullptr};
     int* rows_dev = nullptr;
-    float* ybuf = nullptr;
     float* loss_part = nullptr;
     int n_part = 0;
     float* loss_hist = nullptr;
@@ -521,7 +579,7 @@ namespace {
 
 void free_all(synax_surrogate_t* s) {
     void* ptrs[] = {s->W, s->dW, s->mW, s->vW, s->b, s->db, s->mb, s->vb, s->Wb, s->Wt, s->lo, s->inv2, s->mean,
-                    s->rows_dev, s->ybuf, s->loss_part, s->loss_hist, s->t_dev, s->adam_coef, s->err, s->eD0, s->eD1,
+                    s->rows_dev, s->loss_part, s->loss_hist, s->t_dev, s->adam_coef, s->err, s->eD0, s->eD1,
                     s->sign_dev, s->basis_rows_dev, s->S, s->S_lo, s->maps, s->mhi, s->mlo, s->ctrue, s->ds_theta,
                     s->ds_y};
     for (void* p : ptrs)
@@ -538,7 +596,7 @@ void free_all(synax_surrogate_t* s) {
     if (s->ev_join) cudaEventDestroy(s->ev_join);
 }
 
-LayerTable layer_table(const synax_surrogate_t* s, bool with_tiles) {
+LayerTable layer_table(const synax_surrogate_t* s) {
     LayerTable T{};
     T.L = s->L;
     int tiles = 0;
@@ -549,7 +607,7 @@ LayerTable layer_table(const synax_surrogate_t* s, bool with_tiles) {
         T.boff[l] = s->boff[l];
         T.dZt[l] = s->dZt[l];
         T.tile_begin[l] = tiles;
-        if (with_tiles) tiles += ((s->N[l] + 31) / 32) * ((s->K[l] + 31) / 32);
+        tiles += (s->N[l] / 64) * (s->K[l] / 64);
     }
     T.tile_begin[s->L] = tiles;
     return T;
@@ -563,13 +621,14 @@ AdamHyper hyper(const synax_surrogate_t* s) {
     h.beta2 = (float)s->cfg.beta2;
     h.eps = (float)s->cfg.eps;
     h.total_steps = s->cfg.total_steps;
+    h.ln_beta1 = std::log((double)h.beta1);
+    h.ln_beta2 = std::log((double)h.beta2);
     return h;
 }
 
-int refresh_copies(synax_surrogate_t* s, cudaStream_t st, int update) {
-    const LayerTable T = layer_table(s, true);
-    k_adam_weights<<<T.tile_begin[s->L], dim3(32, 8), 0, st>>>(T, s->W, s->dW, s->mW, s->vW, s->Wb, s->Wt,
-                                                               hyper(s), s->adam_coef, update);
+int refresh_copies(synax_surrogate_t* s, cudaStream_t st) {
+    const LayerTable T = layer_table(s);
+    k_refresh_copies<<<T.tile_begin[s->L], 256, 0, st>>>(T, s->W, s->Wb, s->Wt);
     return launch_status();
 }
 
@@ -580,11 +639,14 @@ int refresh_copies(synax_surrogate_t* s, cudaStream_t st, int update) {
     } while (0)
 
 // Forward + MSE + backward of one batch already gathered into X[0] / Xt[0]
-// with target rows in rows_dev; gradients land in dW, db.
-int enqueue_train_pass(synax_surrogate_t* s, const float* target, cudaStream_t st) {
+// with target rows in rows_dev; the weights' gradients land in dW.  The target
+// is normalised on the way in when `raw` (mean, scale of the outputs).  Every
+// product follows another kernel of the chain, whose end its set-up overlaps.
+int enqueue_train_pass(synax_surrogate_t* s, const float* target, bool raw, cudaStream_t st) {
     const int B = s->B, L = s->L;
     for (int l = 0; l < L; ++l) {
         GemmEpiParams ep{};
+        ep.overlap = 1;
         ep.bias = s->b + s->boff[l];
         if (l < L - 1) {
             ep.out_z = s->Z[l];
@@ -599,6 +661,8 @@ int enqueue_train_pass(synax_surrogate_t* s, const float* target, cudaStream_t s
             ep.target = target;
             ep.ld_target = s->n_out;
             ep.target_rows = s->rows_dev;
+            ep.target_mean = raw ? s->mean : nullptr;
+            ep.target_scale = 1.0f / s->scale;
             ep.coef = (float)(2.0 / ((double)B * (double)s->n_out));
             ep.loss_partial = s->loss_part;
             ep.out_bf16 = s->dZ[l];
@@ -611,11 +675,13 @@ int enqueue_train_pass(synax_surrogate_t* s, const float* target, cudaStream_t s
     }
     for (int l = L - 1; l >= 0; --l) {
         GemmEpiParams ep{};
+        ep.overlap = 1;
         ep.out_f32 = s->dW + s->woff[l];
         ep.ld_f32 = s->K[l];
         SX_TRY(gemm_bf16(s->dZt[l], B, s->Xt[l], B, s->N[l], s->K[l], B, EPI_F32, ep, s->err, st));
         if (l > 0) {
             GemmEpiParams eb{};
+            eb.overlap = 1;
             eb.aux = s->Z[l - 1];
             eb.ld_aux = s->N[l - 1];
             eb.out_bf16 = s->dZ[l - 1];
@@ -626,17 +692,45 @@ int enqueue_train_pass(synax_surrogate_t* s, const float* target, cudaStream_t s
                              s->err, st));
         }
     }
-    const LayerTable T = layer_table(s, false);
-    k_bias_grad<<<(s->n_b * 32 + 255) / 256, 256, 0, st>>>(T, B, s->db);
-    return launch_status();
+    return SYNAX_OK;
 }
 
-int enqueue_update(synax_surrogate_t* s, cudaStream_t st) {
-    k_adam_prep<<<1, 32, 0, st>>>(hyper(s), s->t_dev, s->adam_coef);
-    SX_TRY(launch_status());
-    SX_TRY(refresh_copies(s, st, 1));
-    k_adam_bias<<<(s->n_b + 255) / 256, 256, 0, st>>>(s->b, s->db, s->mb, s->vb, s->n_b, hyper(s), s->adam_coef);
-    return launch_status();
+// The step's end: loss, bias gradients and (update) Adam.
+int enqueue_update(synax_surrogate_t* s, int update, float* loss_out, cudaStream_t st) {
+    UpdateArgs a{};
+    a.T = layer_table(s);
+    a.B = s->B;
+    a.W = s->W;
+    a.dW = s->dW;
+    a.mW = s->mW;
+    a.vW = s->vW;
+    a.Wb = s->Wb;
+    a.Wt = s->Wt;
+    a.b = s->b;
+    a.db = s->db;
+    a.mb = s->mb;
+    a.vb = s->vb;
+    a.bias_blocks = (s->n_b + 7) / 8;
+    a.h = hyper(s);
+    a.coef = s->adam_coef;
+    a.update = update;
+    a.loss_part = s->loss_part;
+    a.n_part = s->n_part;
+    a.inv_count = (float)(1.0 / ((double)s->B * s->n_out));
+    a.loss_hist = s->loss_hist;
+    a.loss_out = loss_out;
+    a.t_dev = s->t_dev;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(1 + a.bias_blocks + (update ? a.T.tile_begin[s->L] : 0)));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_update, a);
+    return e == cudaSuccess ? launch_status() : record_cuda_error((int)e);
 }
 
 GatherArgs gather_identity(const synax_surrogate_t* s, const float* theta, int count, bf16* X, bf16* Xt, int* rows_out) {
@@ -820,7 +914,7 @@ int synax_surrogate_create(const synax_surrogate_cfg* cfg, synax_surrogate_t** o
     }
     const long long dmax = s->n_out > c.width ? s->n_out : c.width;
     SX_ALLOC(s->eD0, (long long)E * dmax) SX_ALLOC(s->eD1, (long long)E * dmax)
-    SX_ALLOC(s->rows_dev, B) SX_ALLOC(s->ybuf, (long long)B * s->n_out)
+    SX_ALLOC(s->rows_dev, B)
     s->n_part = gemm_tiles(B, s->n_out, c.width);
     SX_ALLOC(s->loss_part, s->n_part) SX_ALLOC(s->loss_hist, kLossHist)
     SX_ALLOC(s->t_dev, 1) SX_ALLOC(s->adam_coef, 4) SX_ALLOC(s->err, 1)
@@ -865,7 +959,7 @@ int synax_surrogate_create(const synax_surrogate_cfg* cfg, synax_surrogate_t** o
     } else if ((rc = build_sh_basis(c.nside, c.n_basis, s->S, s->S_lo, nullptr)) != SYNAX_OK) {
         return fail(rc);
     }
-    if ((rc = refresh_copies(s, 0, 0)) != SYNAX_OK) return fail(rc);
+    if ((rc = refresh_copies(s, 0)) != SYNAX_OK) return fail(rc);
     e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return fail(record_cuda_error((int)e));
     *out = s;
@@ -906,7 +1000,7 @@ int synax_surrogate_set_params(synax_surrogate_t* s, const float* host, size_t n
     if (e == cudaSuccess) e = cudaMemset(s->t_dev, 0, 4);
     if (e != cudaSuccess) return record_cuda_error((int)e);
     s->t_host = 0;
-    SX_TRY(refresh_copies(s, 0, 0));
+    SX_TRY(refresh_copies(s, 0));
     e = cudaDeviceSynchronize();
     return e == cudaSuccess ? SYNAX_OK : record_cuda_error((int)e);
 }
@@ -965,16 +1059,12 @@ int synax_surrogate_step(synax_surrogate_t* s, const float* theta_dev, const flo
     if (!s || !theta_dev || !coeff_dev || n != s->B || (update != 0 && update != 1)) return SYNAX_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     GatherArgs a = gather_identity(s, theta_dev, s->B, s->X[0], s->Xt[0], s->rows_dev);
+    a.coef = s->adam_coef;
+    a.hyper = hyper(s);
     k_gather_input<<<(s->B + 3) / 4, 128, 0, st>>>(a);
     SX_TRY(launch_status());
-    k_normalize<<<grid_for((long long)s->B * s->n_out), 256, 0, st>>>(coeff_dev, s->B, s->n_out, s->mean,
-                                                                      1.0f / s->scale, s->ybuf);
-    SX_TRY(launch_status());
-    SX_TRY(enqueue_train_pass(s, s->ybuf, st));
-    if (update) SX_TRY(enqueue_update(s, st));
-    k_finalize<<<1, 32, 0, st>>>(s->loss_part, s->n_part, (float)(1.0 / ((double)s->B * s->n_out)), s->loss_hist,
-                                 s->t_dev, update, loss_dev);
-    SX_TRY(launch_status());
+    SX_TRY(enqueue_train_pass(s, coeff_dev, true, st));
+    SX_TRY(enqueue_update(s, update, loss_dev, st));
     s->t_host += update;
     return SYNAX_OK;
 }
@@ -1074,15 +1164,12 @@ int synax_surrogate_train(synax_surrogate_t* s, int n_steps, uint64_t seed, void
         cudaStream_t cs = s->cap;
         cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return record_cuda_error((int)e);
+        a.coef = s->adam_coef;
+        a.hyper = hyper(s);
         k_gather_input<<<(s->B + 3) / 4, 128, 0, cs>>>(a);
         int rc = launch_status();
-        if (rc == SYNAX_OK) rc = enqueue_train_pass(s, s->ds_y, cs);
-        if (rc == SYNAX_OK) rc = enqueue_update(s, cs);
-        if (rc == SYNAX_OK) {
-            k_finalize<<<1, 32, 0, cs>>>(s->loss_part, s->n_part, (float)(1.0 / ((double)s->B * s->n_out)),
-                                         s->loss_hist, s->t_dev, 1, nullptr);
-            rc = launch_status();
-        }
+        if (rc == SYNAX_OK) rc = enqueue_train_pass(s, s->ds_y, false, cs);
+        if (rc == SYNAX_OK) rc = enqueue_update(s, 1, nullptr, cs);
         e = cudaStreamEndCapture(cs, &g);
         if (rc != SYNAX_OK) {
             if (g) cudaGraphDestroy(g);
