@@ -602,7 +602,7 @@ __device__ __forceinline__ void adjoint_cta(const MapParams<R>& P, const AdjPara
                     Q = Ph::add(Q, -f);
                 }
                 R Or = R(0), Oi = R(0), Opr = R(0), Opi = R(0), Odr = R(0), Odi = R(0);
-                if constexpr (sizeof(R) == 4 && NF >= 2) {
+                if constexpr (sizeof(R) == 4 && NF % 2 == 0) {
                     // frequencies in pairs; the pair sums are folded at the end
                     float2 or2 = dup2(0.f), oi2 = dup2(0.f), opr2 = dup2(0.f), opi2 = dup2(0.f);
                     float2 odr2 = dup2(0.f), odi2 = dup2(0.f);
@@ -814,6 +814,10 @@ static inline int launch_adj_model(const MapParams<R>& P, const AdjParams<R>& A,
     const int F = P.n_freq;
     if (F == 1) return launch_adj_nf<MODEL, 1, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
     if (F == 2) return launch_adj_nf<MODEL, 2, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
+    // (three computed as four cost the FP32 march a fourth phase, sine, cosine and rotation per sample)
+    if constexpr (sizeof(R) == 4 && (MODEL == SYNAX_MODEL_JF12 || MODEL == SYNAX_MODEL_WMAP)) {
+        if (F == 3) return launch_adj_nf<MODEL, 3, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
+    }
     if (F <= 4) return launch_adj_nf<MODEL, 4, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
     if (F <= 8) return launch_adj_nf<MODEL, 8, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);
     return launch_adj_nf<MODEL, 16, R>(P, A, gmaps, target, grad, chi2, maps, partial, st);

@@ -163,6 +163,10 @@ static inline int launch_forward_model(const MapParams<R>& P, R* maps, cudaStrea
     const int F = P.n_freq;
     if (F == 1) return launch_lpr<MODEL, 1, R>(P, maps, st);
     if (F == 2) return launch_lpr<MODEL, 2, R>(P, maps, st);
+    // (three computed as four cost the FP32 march a fourth phase, sine, cosine and rotation per sample)
+    if constexpr (sizeof(R) == 4 && (MODEL == SYNAX_MODEL_JF12 || MODEL == SYNAX_MODEL_WMAP)) {
+        if (F == 3) return launch_lpr<MODEL, 3, R>(P, maps, st);
+    }
     if (F <= 4) return launch_lpr<MODEL, 4, R>(P, maps, st);
     if (F <= 8) return launch_lpr<MODEL, 8, R>(P, maps, st);
     return launch_lpr<MODEL, 16, R>(P, maps, st);

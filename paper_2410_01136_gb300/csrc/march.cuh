@@ -267,9 +267,30 @@ __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 
+// The polynomials of sincos_cw on |r| <= pi/4, as element pairs.
+__device__ __forceinline__ void sincos_poly2(float2 r, float2& sn, float2& cs) {
+    const float2 r2 = mul2(r, r);
+    float2 ps = fma2(r2, dup2(2.7557319e-6f), dup2(-1.9841270e-4f));
+    ps = fma2(r2, ps, dup2(8.3333333e-3f));
+    ps = fma2(r2, ps, dup2(-1.6666667e-1f));
+    sn = fma2(mul2(r, r2), ps, r);
+    float2 pc = fma2(r2, dup2(-2.7557319e-7f), dup2(2.4801587e-5f));
+    pc = fma2(r2, pc, dup2(-1.3888889e-3f));
+    pc = fma2(r2, pc, dup2(4.1666667e-2f));
+    pc = fma2(r2, pc, dup2(-0.5f));
+    cs = fma2(r2, pc, dup2(1.0f));
+}
 // sincos_cw of two arguments, the polynomial arithmetic as element pairs.
-__device__ __forceinline__ void sincos_cw2(float2 x, float2& s, float2& c) {
-    if (!(fabsf(x.x) < 3200.0f && fabsf(x.y) < 3200.0f)) {
+// cls: the angle's class (angle_class), uniform over the kernel.  Class 2
+// (|x| < pi/4 for every sample of the map) is the polynomials alone: the
+// reduction would find k = 0 and return the same bits from about 2.3 times
+// the instructions.  Class 1 needs no range check.
+__device__ __forceinline__ void sincos_cw2(float2 x, float cls, float2& s, float2& c) {
+    if (cls > 1.5f) {
+        sincos_poly2(x, s, c);
+        return;
+    }
+    if (cls < 0.5f && !(fabsf(x.x) < 3200.0f && fabsf(x.y) < 3200.0f)) {
         sincos_cw(x.x, &s.x, &c.x);
         sincos_cw(x.y, &s.y, &c.y);
         return;
@@ -280,21 +301,17 @@ __device__ __forceinline__ void sincos_cw2(float2 x, float2& s, float2& c) {
     float2 r = fma2(neg2(k), dup2(1.5703125f), x);
     r = fma2(neg2(k), dup2(4.837512969970703e-4f), r);
     r = fma2(neg2(k), dup2(7.549790126404332e-8f), r);
-    const float2 r2 = mul2(r, r);
-    float2 ps = fma2(r2, dup2(2.7557319e-6f), dup2(-1.9841270e-4f));
-    ps = fma2(r2, ps, dup2(8.3333333e-3f));
-    ps = fma2(r2, ps, dup2(-1.6666667e-1f));
-    const float2 sn = fma2(mul2(r, r2), ps, r);
-    float2 pc = fma2(r2, dup2(-2.7557319e-7f), dup2(2.4801587e-5f));
-    pc = fma2(r2, pc, dup2(-1.3888889e-3f));
-    pc = fma2(r2, pc, dup2(4.1666667e-2f));
-    pc = fma2(r2, pc, dup2(-0.5f));
-    const float2 cs = fma2(r2, pc, dup2(1.0f));
-    const int qa = __float_as_int(t.x) & 3, qb = __float_as_int(t.y) & 3;
-    const float sa = (qa & 1) ? cs.x : sn.x, ca = (qa & 1) ? sn.x : cs.x;
-    const float sb = (qb & 1) ? cs.y : sn.y, cb = (qb & 1) ? sn.y : cs.y;
-    s = make_float2((qa & 2) ? -sa : sa, (qb & 2) ? -sb : sb);
-    c = make_float2(((qa + 1) & 2) ? -ca : ca, ((qb + 1) & 2) ? -cb : cb);
+    float2 sn, cs;
+    sincos_poly2(r, sn, cs);
+    // quadrant: the swap from bit 0 of k, the signs from bit 1 of k and of k + 1 as sign-bit flips
+    const unsigned qa = __float_as_uint(t.x), qb = __float_as_uint(t.y);
+    const float sa = (qa & 1u) ? cs.x : sn.x, ca = (qa & 1u) ? sn.x : cs.x;
+    const float sb = (qb & 1u) ? cs.y : sn.y, cb = (qb & 1u) ? sn.y : cs.y;
+    const unsigned m = 0x80000000u;
+    s = make_float2(__uint_as_float(__float_as_uint(sa) ^ ((qa << 30) & m)),
+                    __uint_as_float(__float_as_uint(sb) ^ ((qb << 30) & m)));
+    c = make_float2(__uint_as_float(__float_as_uint(ca) ^ (((qa << 30) + 0x40000000u) & m)),
+                    __uint_as_float(__float_as_uint(cb) ^ (((qb << 30) + 0x40000000u) & m)));
 }
 
 // Two double-float sums of one double-float a with floats b.x, b.y
@@ -1027,7 +1044,7 @@ template <> struct Model<SYNAX_MODEL_WMAP_STACK> {
             R sp, cp, sc, cc;
             if constexpr (sizeof(R) == 4) {
                 float2 sv, cv;
-                sincos_cw2(make_float2(psi, chi), sv, cv);
+                sincos_cw2(make_float2(psi, chi), fminf(m[mc::S_CLASS + 2 * k], m[mc::S_CLASS + 2 * k + 1]), sv, cv);
                 sp = sv.x; cp = cv.x; sc = sv.y; cc = cv.y;
             } else {
                 F::sincos(psi, &sp, &cp);
@@ -1557,8 +1574,8 @@ __device__ __forceinline__ void wmap_eval(const float* m, float2 x, float2 y, fl
     const float2 env = expf2(neg2(add2(mulc(rho, 0.125), az)));
     const float2 amp = mul2(dup2(m[mc::W_B0]), env);
     float2 sp, cp, sc, cc;
-    sincos_cw2(psi, sp, cp);
-    sincos_cw2(chi, sc, cc);
+    sincos_cw2(psi, m[mc::W_CLASS], sp, cp);
+    sincos_cw2(chi, m[mc::W_CLASS + 1], sc, cc);
     const float2 br = mul2(mul2(amp, cp), cc), bp = mul2(mul2(amp, sp), cc);
     B[0] = add2(fma2(br, c, neg2(mul2(bp, s))), dup2(m[mc::W_BUX]));
     B[1] = fma2(br, s, mul2(bp, c));
@@ -1618,8 +1635,8 @@ __device__ __forceinline__ void stack_eval(const float* m, float2 x, float2 y, f
         const float2 psi = f2(in_a ? fmaf(q[2], lnr8.x, q[1]) : 0.0f, in_b ? fmaf(q[2], lnr8.y, q[1]) : 0.0f);
         const float2 chi = f2(in_a ? q[3] * th.x : 0.0f, in_b ? q[3] * th.y : 0.0f);
         float2 sp, cp, sc, cc;
-        sincos_cw2(psi, sp, cp);
-        sincos_cw2(chi, sc, cc);
+        sincos_cw2(psi, m[mc::S_CLASS + 2 * k], sp, cp);
+        sincos_cw2(chi, m[mc::S_CLASS + 2 * k + 1], sc, cc);
         const float2 ur = mul2(cp, cc), up = mul2(sp, cc);
         const float2 hi = dup2(m[mc::S_WB + k]), lo = dup2(m[mc::S_WB_LO + k]);
         const float2 u0 = fma2(ur, c, neg2(mul2(up, s)));
@@ -1923,7 +1940,7 @@ __device__ __forceinline__ void march_lane(const MapParams<R>& P, const R* s_arm
             s_n = fma(P.w_own, e.f, S);
             S = Ph::add(S, e.f);
         }
-        if constexpr (sizeof(R) == 4 && NF >= 2) {
+        if constexpr (sizeof(R) == 4 && NF % 2 == 0) {
             // frequencies in pairs: (pc + i ps) e^{i phi} for two at once.
             // All NF are computed; those beyond n_freq have phase constant 0
             // and are never stored.
@@ -1952,7 +1969,7 @@ __device__ __forceinline__ void march_lane(const MapParams<R>& P, const R* s_arm
         // chunk at the end: harmless, its state is not used again)
         if constexpr (MODEL == SYNAX_MODEL_JF12) trk.step(+1);
     }
-    if constexpr (sizeof(R) == 4 && NF >= 2) {
+    if constexpr (sizeof(R) == 4 && NF % 2 == 0) {
 #pragma unroll
         for (int k = 0; k < NF; k += 2) {
             zr[k] = zr2[k >> 1].x;

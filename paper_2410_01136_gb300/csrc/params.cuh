@@ -122,6 +122,9 @@ SYNAX_HD inline void fill_theta(int model, const double* th, const double* freq_
         M.m[mc::W_N0OBS] = R(th[5]);
         M.m[mc::W_NE0] = R(th[7]);
         M.m[mc::W_NE0_LO] = lo_part<R>(th[7]);
+        // |ln(rho/8)| <= ln(8/3) = 0.9809 and |tanh z| <= 1 in the field's range
+        M.m[mc::W_CLASS] = R(angle_class(::fabs(th[1]) + 0.981 * ::fabs(th[2])));
+        M.m[mc::W_CLASS + 1] = R(angle_class(::fabs(th[3])));
         break;
     case SYNAX_MODEL_JF12:
         for (int k = 0; k < 8; ++k) M.m[mc::J_B + k] = R(th[k]);
@@ -158,6 +161,8 @@ SYNAX_HD inline void fill_theta(int model, const double* th, const double* freq_
             const double wb = stack_w(k) * th[4 * k];
             M.m[mc::S_WB + k] = R(wb);
             M.m[mc::S_WB_LO + k] = lo_part<R>(wb);
+            M.m[mc::S_CLASS + 2 * k] = R(angle_class(::fabs(th[4 * k + 1]) + 0.981 * ::fabs(th[4 * k + 2])));
+            M.m[mc::S_CLASS + 2 * k + 1] = R(angle_class(::fabs(th[4 * k + 3])));
         }
         break;
     case SYNAX_MODEL_GRID:
