@@ -82,12 +82,15 @@ def eval_fields(prob, pos, t, stream=None):
     return out
 
 
-def adjoint_workspace_bytes(prob) -> int:
-    s = problem_struct(prob)
+def _adjoint_workspace_bytes(s) -> int:
     n = ctypes.c_size_t(0)
     check(lib().synax_adjoint_workspace_bytes(ctypes.byref(s), ctypes.byref(n)),
           "synax_adjoint_workspace_bytes")
     return int(n.value)
+
+
+def adjoint_workspace_bytes(prob) -> int:
+    return _adjoint_workspace_bytes(problem_struct(prob))
 
 
 def adjoint(prob, gmaps=None, target=None, sigma: float = 1.0, maps_out=None, workspace=None,
@@ -105,12 +108,12 @@ def adjoint(prob, gmaps=None, target=None, sigma: float = 1.0, maps_out=None, wo
     _check_map_tensor(torch, seed, prob, "gmaps" if gmaps is not None else "target")
     if maps_out is not None:
         _check_map_tensor(torch, maps_out, prob, "maps_out")
-    nbytes = adjoint_workspace_bytes(prob)
+    s = problem_struct(prob)
+    nbytes = _adjoint_workspace_bytes(s)
     if workspace is None:
         workspace = torch.empty(max(nbytes, 1), dtype=torch.uint8, device="cuda")
     grad = torch.empty(len(prob.theta), dtype=torch.float64, device="cuda")
     chi2 = torch.empty(1, dtype=torch.float64, device="cuda") if target is not None else None
-    s = problem_struct(prob)
     check(lib().synax_adjoint(
         ctypes.byref(s),
         ctypes.c_void_p(gmaps.data_ptr() if gmaps is not None else 0),
