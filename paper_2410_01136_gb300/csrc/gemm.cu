@@ -102,24 +102,35 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // reciprocal and one exponential on the SFU for both.  Phi is off by at most
 // ~1e-7 absolute, far below the BF16 rounding (2^-9 relative) of the
 // activations these feed.
-struct NormalCdf {
-    float Phi, g;
+// Two arguments at a time: sm_100 executes two FP32 operations of a thread
+// per paired instruction (rounded as the scalar ones), and the epilogue warps
+// of the GELU layers are limited by what they issue.
+struct NormalCdf2 {
+    float2 Phi, g;
 };
-__device__ __forceinline__ NormalCdf normal_cdf(float z) {
-    const float x = fabsf(z) * 0.70710678118654752f;
-    float t, g;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, x, 1.0f)));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(g) : "f"(z * z * -0.72134752044448170f));   // -log2(e) / 2
-    const float P =
-        t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f),
-                 0.254829592f);
-    const float q = 0.5f * P * g;       // Phi(-|z|)
-    return {z >= 0.0f ? 1.0f - q : q, g};
+__device__ __forceinline__ float2 bcast2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ NormalCdf2 normal_cdf2(float2 z) {
+    const float2 x = __fmul2_rn(make_float2(fabsf(z.x), fabsf(z.y)), bcast2(0.70710678118654752f));
+    const float2 d = __ffma2_rn(bcast2(0.3275911f), x, bcast2(1.0f));
+    const float2 e = __fmul2_rn(__fmul2_rn(z, z), bcast2(-0.72134752044448170f));   // -log2(e) / 2
+    float2 t, g;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.x) : "f"(d.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t.y) : "f"(d.y));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(g.x) : "f"(e.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(g.y) : "f"(e.y));
+    float2 P = __ffma2_rn(t, bcast2(1.061405429f), bcast2(-1.453152027f));
+    P = __ffma2_rn(t, P, bcast2(1.421413741f));
+    P = __ffma2_rn(t, P, bcast2(-0.284496736f));
+    P = __fmul2_rn(t, __ffma2_rn(t, P, bcast2(0.254829592f)));
+    const float2 h = __fmul2_rn(bcast2(0.5f), P);
+    const float2 q = __fmul2_rn(h, g);                                               // Phi(-|z|)
+    const float2 u = __fadd2_rn(bcast2(1.0f), make_float2(-q.x, -q.y));
+    return {make_float2(z.x >= 0.0f ? u.x : q.x, z.y >= 0.0f ? u.y : q.y), g};
 }
-__device__ __forceinline__ float gelu_f(float z) { return z * normal_cdf(z).Phi; }
-__device__ __forceinline__ float gelu_grad_f(float z) {
-    const NormalCdf n = normal_cdf(z);
-    return fmaf(z * 0.39894228040143268f, n.g, n.Phi);   // Phi(z) + z phi(z)
+__device__ __forceinline__ float2 gelu2(float2 z) { return __fmul2_rn(z, normal_cdf2(z).Phi); }
+__device__ __forceinline__ float2 gelu_grad2(float2 z) {
+    const NormalCdf2 n = normal_cdf2(z);
+    return __ffma2_rn(__fmul2_rn(z, bcast2(0.39894228040143268f)), n.g, n.Phi);       // Phi(z) + z phi(z)
 }
 
 
@@ -195,20 +206,24 @@ __device__ __forceinline__ void epilogue16(const GemmEpiParams& ep, const float*
             }
         }
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            float x = v[i];
+        for (int i = 0; i < 16; i += 2) {
+            const float2 x = make_float2(v[i], v[i + 1]);
+            float2 y;
             if constexpr (EPI == EPI_BIAS_GELU) {
-                const float z = x + b[i];
-                z16[i] = z;
-                x = gelu_f(z);
+                const float2 z = __fadd2_rn(x, make_float2(b[i], b[i + 1]));
+                z16[i] = z.x;
+                z16[i + 1] = z.y;
+                y = gelu2(z);
             } else if constexpr (EPI == EPI_GELU_BWD) {
-                x *= gelu_grad_f(a[i]);
+                y = __fmul2_rn(x, gelu_grad2(make_float2(a[i], a[i + 1])));
             } else {   // EPI_MSE
-                const float d = x + b[i] - t[i];
-                if (i < nv) sq = fmaf(d, d, sq);
-                x = ep.coef * d;
+                const float2 d = __fadd2_rn(__fadd2_rn(x, make_float2(b[i], b[i + 1])), make_float2(-t[i], -t[i + 1]));
+                if (i < nv) sq = fmaf(d.x, d.x, sq);
+                if (i + 1 < nv) sq = fmaf(d.y, d.y, sq);
+                y = __fmul2_rn(bcast2(ep.coef), d);
             }
-            r[i] = x;
+            r[i] = y.x;
+            r[i + 1] = y.y;
         }
         if constexpr (EPI == EPI_BIAS_GELU) {
             if (keep_z) {
