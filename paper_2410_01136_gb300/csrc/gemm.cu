@@ -30,6 +30,10 @@
 //                        area; other outputs are vectorised row stores
 //                        (coalesced transposed stores).
 // With two accumulators the MMAs of tile i+1 run while tile i is stored.
+// Products with many rows and a long K run on pairs of CTAs (clusters of 2,
+// cta_group::2): a 256 x 256 tile, of which each CTA loads 128 rows of A and
+// 128 of B and keeps 128 rows of the accumulator; CTA 0 issues the MMAs, and
+// its barriers collect both CTAs' loads and accumulator releases.
 // Every mbarrier wait gives up after ~1 s of SM clocks and sets *err; each
 // role then stops, the MMA issuer waits (bounded) for its issued MMAs, the
 // producer for its loads in flight, and the CTA frees its TMEM and returns.
@@ -56,9 +60,12 @@ constexpr int kGemmBK = 64;
 // columns; the FP32 epilogues keep 4, one per quadrant, which their TMA-store
 // staging chunks (128 rows x 32 columns) are laid out for, and so do 32-column
 // tiles, which are one block wide.
+constexpr bool gemm_f32_out(int epi) {
+    return epi == EPI_F32 || epi == EPI_BIAS_F32 || epi == EPI_AFFINE || epi == EPI_SCALE_ACC;
+}
 template <int BN, int EPI>
 constexpr int gemm_epi_warps() {
-    return BN > 32 && (EPI == EPI_BIAS_GELU || EPI == EPI_GELU_BWD || EPI == EPI_MSE) ? 8 : 4;
+    return BN > 32 && !gemm_f32_out(EPI) ? 8 : 4;
 }
 template <int BN, int EPI>
 constexpr int gemm_threads() {
@@ -66,15 +73,19 @@ constexpr int gemm_threads() {
 }
 constexpr long long kWaitCycles = 2000000000LL;   // ~1 s at 2 GHz
 
-template <int BN, int EPI = EPI_F32>
+// PAIR: two CTAs of a cluster share a 256 x BN tile (cta_group::2); each loads
+// its 128 rows of A and half of B's rows.
+template <int BN, int EPI = EPI_F32, bool PAIR = false>
 struct GemmCfg {
     // The BF16 activations of the GELU and GELU' epilogues leave through TMA
     // stores from per-warp 32 x 32 staging blocks (8 epilogue warps x 2 KB,
-    // BN = 128); one pipeline stage fewer makes room for them.
-    static constexpr bool BF16_STAGE = BN == 128 && (EPI == EPI_BIAS_GELU || EPI == EPI_GELU_BWD);
-    static constexpr int ST = BN == 256 ? 4 : (BF16_STAGE ? 5 : 6);   // pipeline stages
+    // BN = 128 and pairs); one pipeline stage fewer makes room for them.
+    static constexpr bool BF16_STAGE = (BN == 128 || PAIR) && (EPI == EPI_BIAS_GELU || EPI == EPI_GELU_BWD);
+    static constexpr int TM = PAIR ? 2 * kGemmBM : kGemmBM;            // rows of a tile
+    static constexpr int B_ROWS = PAIR ? BN / 2 : BN;                  // rows of B that a CTA loads
+    static constexpr int ST = BN == 256 && !PAIR ? 4 : (BF16_STAGE ? 5 : 6);   // pipeline stages
     static constexpr uint32_t A_BYTES = kGemmBM * kGemmBK * 2;
-    static constexpr uint32_t B_BYTES = BN * kGemmBK * 2;
+    static constexpr uint32_t B_BYTES = B_ROWS * kGemmBK * 2;
     static constexpr uint32_t TMEM_COLS = 2 * BN;                      // two accumulators
     static constexpr uint32_t STG_BYTES = kGemmBM * 32 * 4;                 // one 128 x 32 FP32 chunk
     static constexpr uint32_t BF16_BLOCK = 32 * 32 * 2;                     // one warp's 32 x 32 BF16 block
@@ -271,12 +282,12 @@ __device__ __forceinline__ void epilogue16(const GemmEpiParams& ep, const float*
     }
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool PAIR>
 __global__ void __launch_bounds__(gemm_threads<BN, EPI>(), 1)
 k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
             const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmD, int M, int N, int K,
             GemmEpiParams ep, int* err) {
-    using C = GemmCfg<BN, EPI>;
+    using C = GemmCfg<BN, EPI, PAIR>;
     constexpr int ST = C::ST;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -295,6 +306,9 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    // a pair: CTA 0 issues the MMAs of both and collects both CTAs' loads and
+    // hand-offs on its own barriers
+    const uint32_t rank = PAIR ? tc::cluster_rank() : 0u;
     // The set-up below touches no global memory, so it may run while the
     // previous kernel of the stream finishes, and the next one's while this
     // one runs (every CTA of this grid is resident by then).
@@ -308,20 +322,26 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&acc_full[b], 1);
-            tc::mbar_init(&acc_empty[b], EW);
+            tc::mbar_init(&acc_empty[b], PAIR ? 2 * EW : EW);
         }
         tc::mbar_init(drain, 1);
         tc::fence_mbar_init();
     }
-    if (warp == 1) tc::tmem_alloc(tmem_slot, C::TMEM_COLS);
+    if (warp == 1) {
+        if constexpr (PAIR) tc::tmem_alloc_pair(tmem_slot, C::TMEM_COLS);
+        else tc::tmem_alloc(tmem_slot, C::TMEM_COLS);
+    }
     tc::fence_before_sync();
     __syncthreads();
+    if constexpr (PAIR) tc::cluster_sync();       // both CTAs' barriers are ready
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
     tc::grid_dependency_wait();
 
     const int tiles_n = (N + BN - 1) / BN;
-    const int tiles = tiles_n * ((M + kGemmBM - 1) / kGemmBM);
+    const int tiles = tiles_n * ((M + C::TM - 1) / C::TM);
+    const int first = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
+    const int stride = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
     const int KT = K / kGemmBK;
     bool ok = true;
     float sq = 0.0f;
@@ -329,30 +349,38 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     if (warp == 0) {
         if (lane == 0) {
             int it = 0;   // stage loads issued
-            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-                const int m0 = (t / tiles_n) * kGemmBM, n0 = (t % tiles_n) * BN;
+            for (int t = first; t < tiles && ok; t += stride) {
+                const int m0 = (t / tiles_n) * C::TM + (int)rank * kGemmBM, n0 = (t % tiles_n) * BN;
                 for (int kt = 0; kt < KT; ++kt, ++it) {
                     const int s = it % ST;
                     if (it >= ST && !mbar_wait_clock(&empty[s], ((it / ST) - 1) & 1)) {
                         ok = false;
                         break;
                     }
-                    tc::mbar_expect_tx(&full[s], C::A_BYTES + C::B_BYTES);
-                    tc::tma_load_2d(sA + s * C::A_BYTES, &tmA, &full[s], kt * kGemmBK, m0);
-                    tc::tma_load_2d(sB + s * C::B_BYTES, &tmB, &full[s], kt * kGemmBK, n0);
+                    if constexpr (PAIR) {
+                        if (rank == 0) tc::mbar_expect_tx(&full[s], 2 * (C::A_BYTES + C::B_BYTES));
+                        const uint32_t bar = tc::map_to_rank(&full[s], 0);
+                        tc::tma_load_2d_pair(sA + s * C::A_BYTES, &tmA, bar, kt * kGemmBK, m0);
+                        tc::tma_load_2d_pair(sB + s * C::B_BYTES, &tmB, bar, kt * kGemmBK, n0 + (int)rank * C::B_ROWS);
+                    } else {
+                        tc::mbar_expect_tx(&full[s], C::A_BYTES + C::B_BYTES);
+                        tc::tma_load_2d(sA + s * C::A_BYTES, &tmA, &full[s], kt * kGemmBK, m0);
+                        tc::tma_load_2d(sB + s * C::B_BYTES, &tmB, &full[s], kt * kGemmBK, n0);
+                    }
                 }
             }
             if (!ok) {
-                // let the loads still in flight (the last min(it, ST)) land
+                // let the loads still in flight (the last min(it, ST)) land (a
+                // pair's CTA 1, whose loads report to CTA 0, waits out the limit here)
                 for (int j = it > ST ? it - ST : 0; j < it; ++j) mbar_wait_clock(&full[j % ST], (j / ST) & 1);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(kGemmBM, BN);
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = tc::idesc_bf16_f32(C::TM, BN);
             int it = 0, j = 0;
             bool issued = false;
-            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++j) {
+            for (int t = first; t < tiles && ok; t += stride, ++j) {
                 const int buf = j & 1;
                 if (j >= 2 && !mbar_wait_clock(&acc_empty[buf], ((j >> 1) - 1) & 1)) {
                     ok = false;
@@ -370,18 +398,23 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     const uint32_t a0 = tc::smem_u32(sA + s * C::A_BYTES);
                     const uint32_t b0 = tc::smem_u32(sB + s * C::B_BYTES);
 #pragma unroll
-                    for (int kk = 0; kk < kGemmBK / 16; ++kk)
-                        tc::mma_bf16(acc, tc::desc_kmajor_sw128(a0 + kk * 32), tc::desc_kmajor_sw128(b0 + kk * 32),
-                                     idesc, (kt | kk) != 0 ? 1u : 0u);
+                    for (int kk = 0; kk < kGemmBK / 16; ++kk) {
+                        const uint64_t da = tc::desc_kmajor_sw128(a0 + kk * 32), db = tc::desc_kmajor_sw128(b0 + kk * 32);
+                        if constexpr (PAIR) tc::mma_bf16_pair(acc, da, db, idesc, (kt | kk) != 0 ? 1u : 0u);
+                        else tc::mma_bf16(acc, da, db, idesc, (kt | kk) != 0 ? 1u : 0u);
+                    }
                     issued = true;
-                    tc::mma_commit(&empty[s]);
+                    if constexpr (PAIR) tc::mma_commit_pair(&empty[s]);
+                    else tc::mma_commit(&empty[s]);
                 }
                 if (!ok) break;
-                tc::mma_commit(&acc_full[buf]);
+                if constexpr (PAIR) tc::mma_commit_pair(&acc_full[buf]);
+                else tc::mma_commit(&acc_full[buf]);
             }
             if (issued) {
                 // every MMA of this thread has completed once drain fires
-                tc::mma_commit(drain);
+                if constexpr (PAIR) tc::mma_commit_pair(drain);
+                else tc::mma_commit(drain);
                 if (!mbar_wait_clock(drain, 0)) ok = false;
             }
         }
@@ -394,7 +427,7 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         int j = 0;
         int stg = 0;       // staging chunks used (TMA-store path)
         int zblk = 0;      // staged GELU / GELU' blocks stored by this warp
-        for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++j) {
+        for (int t = first; t < tiles; t += stride, ++j) {
             const int buf = j & 1;
             // all EW epilogue warps agree (they share named barriers below):
             // every one of them reaches this reduction each tile, waited or not
@@ -405,7 +438,7 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 break;
             }
             tc::fence_after_sync();
-            const int m0 = (t / tiles_n) * kGemmBM, n0 = (t % tiles_n) * BN;
+            const int m0 = (t / tiles_n) * C::TM + (int)rank * kGemmBM, n0 = (t % tiles_n) * BN;
             const int row = m0 + q * 32 + lane;
             const bool row_ok = row < M;
             long long trow = row;
@@ -413,7 +446,7 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 if (row_ok && ep.target_rows) trow = ep.target_rows[row];
             }
             const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN);
-            constexpr bool kF32Out = EPI == EPI_F32 || EPI == EPI_BIAS_F32 || EPI == EPI_AFFINE || EPI == EPI_SCALE_ACC;
+            constexpr bool kF32Out = gemm_f32_out(EPI);
             static_assert(!kF32Out || EW == 4, "the TMA-store staging serves one warp per lane quadrant");
             if (kF32Out && ep.tma_store) {
                 // 32 columns at a time through a swizzled staging chunk and a TMA store
@@ -536,7 +569,7 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                             }
                             tc::fence_proxy_async_smem();
                             __syncwarp();
-                            if (lane == 0) {
+                            if (lane == 0 && m0 < M) {
                                 // n0 + c is a multiple of 32: 128 bytes (FP32) and 64 bytes (BF16)
                                 if (zst) tc::tma_store_2d(&tmC, zslot, n0 + c, m0 + q * 32);
                                 if (bst) tc::tma_store_2d(&tmD, bslot, n0 + c, m0 + q * 32);
@@ -550,7 +583,10 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
             tc::fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+            if (lane == 0) {
+                if constexpr (PAIR) tc::mbar_arrive_remote(tc::map_to_rank(&acc_empty[buf], 0));
+                else mbar_arrive(&acc_empty[buf]);
+            }
         }
         if constexpr (EPI == EPI_MSE) {
 #pragma unroll
@@ -574,9 +610,12 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             ep.loss_partial[blockIdx.x] = l;
         }
     }
+    // neither CTA of a pair leaves while the other may signal it or use its operands
+    if constexpr (PAIR) tc::cluster_sync();
     if (warp == 1) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, C::TMEM_COLS);
+        if constexpr (PAIR) tc::tmem_dealloc_pair(tmem, C::TMEM_COLS);
+        else tc::tmem_dealloc(tmem, C::TMEM_COLS);
     }
 }
 
@@ -639,6 +678,43 @@ static int gemm_bn_for(int M, int N, int K, int sms) {
     return bn;
 }
 
+// Tile width and whether CTA pairs share 256 x 256 tiles.
+// Single CTAs with an FP32 output (its 128-row staging chunks keep the
+// epilogue light) and two waves of tiles or more take 256 columns instead of
+// 128: a 128 x 256 tile takes in 768 KB of operands per 2 x 128 x 256 x K flop
+// against 512 KB per half the work, and the SMs' operand bandwidth is what a
+// 128-column tile runs out of at K ~ 1024 (16384 x 1024 x 1024: 40.3 against 48.1 us).
+// A pair takes in 128 + 128 rows of operands per K tile and CTA for 128 x 256
+// products, against 128 + 256 of a single CTA or two tiles of 128 + 128, so it
+// is taken where waves x bytes is smaller, for the BF16 outputs with a K long
+// enough that the operands bound the tile and not its epilogue: GELU from
+// K = 1024 (16384 x 1024 x 1024: 47.7 against 52.6 us; K = 64: 39.4 against
+// 32.7), GELU' from 2048 (16384 x 1024 x 9216: 197 against 216 us; x 1024,
+// where its pre-activation is read in the epilogue: 54 against 50), MSE as
+// GELU.  FP32 outputs gain nothing: their stores bound them (16384 x 9216 x
+// 1024: 217 against 219 us as pairs, x 64 124 against 91).
+struct GemmShape {
+    int bn;
+    bool pair;
+};
+static GemmShape gemm_shape(int M, int N, int K, int epi, int sms, int clusters) {
+    GemmShape s{gemm_bn_for(M, N, K, sms), false};
+    const bool f32_out = gemm_f32_out(epi);
+    const long long rows = (M + kGemmBM - 1) / kGemmBM;
+    if (f32_out && s.bn == 128 && N >= 1024 && rows * ((N + 255) / 256) >= 2LL * sms) s.bn = 256;
+    if (clusters > 0 && !f32_out && N >= 256 && K >= (epi == EPI_GELU_BWD ? 2048 : 1024)) {
+        const long long tiles = rows * ((N + s.bn - 1) / s.bn);
+        const long long pairs = (long long)((M + 255) / 256) * ((N + 255) / 256);
+        if ((pairs + clusters - 1) / clusters * 256 < (tiles + sms - 1) / sms * (kGemmBM + s.bn)) s = {256, true};
+    }
+    return s;
+}
+static int gemm_ctas(const GemmShape& s, int M, int N, int sms, int clusters) {
+    const int tm = s.pair ? 2 * kGemmBM : kGemmBM;
+    const int tiles = ((N + s.bn - 1) / s.bn) * ((M + tm - 1) / tm);
+    return s.pair ? 2 * (tiles < clusters ? tiles : clusters) : (tiles < sms ? tiles : sms);
+}
+
 namespace {
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -685,10 +761,10 @@ int sm_count() {
     return n;
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool PAIR = false>
 cudaError_t set_smem_attr() {
-    return cudaFuncSetAttribute(k_gemm_bf16<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)GemmCfg<BN, EPI>::SMEM);
+    return cudaFuncSetAttribute(k_gemm_bf16<BN, EPI, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)GemmCfg<BN, EPI, PAIR>::SMEM);
 }
 
 template <int EPI>
@@ -697,7 +773,33 @@ cudaError_t set_smem_attrs() {
     if (e == cudaSuccess) e = set_smem_attr<64, EPI>();
     if (e == cudaSuccess) e = set_smem_attr<128, EPI>();
     if (e == cudaSuccess) e = set_smem_attr<256, EPI>();
+    if constexpr (!gemm_f32_out(EPI)) {
+        if (e == cudaSuccess) e = set_smem_attr<256, EPI, true>();
+    }
     return e;
+}
+
+// Pairs of CTAs that the device holds at once (one CTA per SM), 0 if none.
+int pair_clusters() {
+    static int n = 0;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        if (set_smem_attr<256, EPI_MSE, true>() == cudaSuccess) {
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)(2 * (sm_count() / 2)));
+            cfg.blockDim = dim3((unsigned)gemm_threads<256, EPI_MSE>());
+            cfg.dynamicSmemBytes = GemmCfg<256, EPI_MSE, true>::SMEM;
+            cudaLaunchAttribute attr{};
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = 2;
+            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&n, k_gemm_bf16<256, EPI_MSE, true>, &cfg) != cudaSuccess) n = 0;
+        }
+        cudaGetLastError();
+    });
+    return n;
 }
 
 // 2-D FP32 tensor map of an output [rows][ld], box 32 x box_rows, 128-byte swizzle.
@@ -728,17 +830,17 @@ int make_bf16_out_map(CUtensorMap* map, const void* base, int rows, int cols, in
     return r == CUDA_SUCCESS ? SYNAX_OK : SYNAX_EINVAL;
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, bool PAIR = false>
 int launch_gemm_t(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, int K, const GemmEpiParams& ep_in,
                   int* err, cudaStream_t st) {
-    const int tiles = ((N + BN - 1) / BN) * ((M + kGemmBM - 1) / kGemmBM);
-    const int grid = tiles < sm_count() ? tiles : sm_count();
+    using C = GemmCfg<BN, EPI, PAIR>;
+    const int grid = gemm_ctas({BN, PAIR}, M, N, sm_count(), PAIR ? pair_clusters() : 0);
     GemmEpiParams ep = ep_in;
     ep.status = device_status_word();
     CUtensorMap mc;
     std::memset(&mc, 0, sizeof mc);
     ep.tma_store = 0;
-    constexpr bool kF32Out = EPI == EPI_F32 || EPI == EPI_BIAS_F32 || EPI == EPI_AFFINE || EPI == EPI_SCALE_ACC;
+    constexpr bool kF32Out = gemm_f32_out(EPI);
     if (kF32Out && !(EPI == EPI_SCALE_ACC && ep.accumulate) && ep.out_f32 &&
         ((uintptr_t)ep.out_f32 & 15) == 0 && (ep.ld_f32 & 3) == 0 &&
         make_out_map(&mc, ep.out_f32, M, N, ep.ld_f32) == SYNAX_OK)
@@ -752,20 +854,29 @@ int launch_gemm_t(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, in
     CUtensorMap md;
     std::memset(&md, 0, sizeof md);
     ep.tma_store_bf16 = 0;
-    if (GemmCfg<BN, EPI>::BF16_STAGE && ep.out_bf16 && !ep.out_bf16_t && ((uintptr_t)ep.out_bf16 & 15) == 0 &&
+    if (C::BF16_STAGE && ep.out_bf16 && !ep.out_bf16_t && ((uintptr_t)ep.out_bf16 & 15) == 0 &&
         (ep.ld_bf16 & 7) == 0 && make_bf16_out_map(&md, ep.out_bf16, M, N, ep.ld_bf16) == SYNAX_OK)
         ep.tma_store_bf16 = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)gemm_threads<BN, EPI>());
-    cfg.dynamicSmemBytes = GemmCfg<BN, EPI>::SMEM;
+    cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = st;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = ep.overlap ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_bf16<BN, EPI>, ma, mb, mc, md, M, N, K, ep, err);
+    cudaLaunchAttribute attr[2]{};
+    int n_attr = 0;
+    if (ep.overlap) {
+        attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (PAIR) {
+        attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+        attr[n_attr].val.clusterDim.x = 2;
+        attr[n_attr].val.clusterDim.y = 1;
+        attr[n_attr++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = (unsigned)n_attr;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_bf16<BN, EPI, PAIR>, ma, mb, mc, md, M, N, K, ep, err);
     if (e == cudaSuccess) e = cudaGetLastError();
     return e == cudaSuccess ? SYNAX_OK : record_cuda_error((int)e);
 }
@@ -774,17 +885,14 @@ template <int EPI>
 int launch_gemm_bn(const CUtensorMap& ma, const void* B, int N, int K, int ldb, int M, const GemmEpiParams& ep,
                    int* err, cudaStream_t st) {
     CUtensorMap mb;
-    int bn = gemm_bn_for(M, N, K, sm_count());
-    // FP32 outputs (their 128-row staging chunks keep the epilogue light): a
-    // 128 x 256 tile fetches 768 KB of operands per 2 x 128 x 256 x K flop
-    // against 512 KB per half the work at 128 columns, and the SMs' operand
-    // bandwidth is what a 128-column tile runs out of at K ~ 1024
-    // (16384 x 1024 x 1024: 40.3 against 48.1 us).  Only with two waves of
-    // tiles or more, so that smaller products keep enough CTAs.
-    constexpr bool kF32Out = EPI == EPI_F32 || EPI == EPI_BIAS_F32 || EPI == EPI_AFFINE || EPI == EPI_SCALE_ACC;
-    if (kF32Out && bn == 128 && N >= 1024 &&
-        (long long)((M + kGemmBM - 1) / kGemmBM) * ((N + 255) / 256) >= 2LL * sm_count())
-        bn = 256;
+    const GemmShape shape = gemm_shape(M, N, K, EPI, sm_count(), pair_clusters());
+    const int bn = shape.bn;
+    if constexpr (!gemm_f32_out(EPI)) {
+        if (shape.pair) {
+            if (make_map(&mb, B, N, K, ldb, GemmCfg<256, EPI, true>::B_ROWS) != SYNAX_OK) return SYNAX_EINVAL;
+            return launch_gemm_t<256, EPI, true>(ma, mb, M, N, K, ep, err, st);
+        }
+    }
     if (bn == 256) {
         if (make_map(&mb, B, N, K, ldb, 256) != SYNAX_OK) return SYNAX_EINVAL;
         return launch_gemm_t<256, EPI>(ma, mb, M, N, K, ep, err, st);
@@ -823,9 +931,8 @@ int gemm_init() {
 int device_sm_count() { return sm_count(); }
 
 int gemm_tiles(int M, int N, int K) {
-    const int bn = gemm_bn_for(M, N, K, sm_count());
-    const int tiles = ((N + bn - 1) / bn) * ((M + kGemmBM - 1) / kGemmBM);
-    return tiles < sm_count() ? tiles : sm_count();
+    const int clusters = pair_clusters();
+    return gemm_ctas(gemm_shape(M, N, K, EPI_MSE, sm_count(), clusters), M, N, sm_count(), clusters);
 }
 
 // C = A[M][K] . B[N][K]^T with the given epilogue.  A, B: BF16 row-major with
