@@ -7,8 +7,8 @@
 // taken apart with integer instructions, the reduction and the polynomial run
 // on unsigned 64-bit fractions (a product's high half is 3 wide integer
 // multiplies and 2 additions), and the result is rounded once to FP64: no
-// FP64 instruction at all.  The FP64 march keeps 85 FP64 instructions per
-// sample (the grid model; pipe 77 % active, issue 34 %).  Measured against
+// FP64 instruction at all.  The FP64 march keeps 73 FP64 instructions per
+// sample (the grid model; pipe 70 % active, issue 35 %).  Measured against
 // CUDA's functions: a map of a 256 x 256 x 64 grid (Nside 64, 512 steps)
 // 14.5 -> 4.0 ms, WMAP-type maps and gradient (Nside 16, 128 steps, 2
 // frequencies) 1.33 -> 0.58 ms (4.2 and 0.64 ms before the lane count followed),
