@@ -373,6 +373,12 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 // let the loads still in flight (the last min(it, ST)) land (a
                 // pair's CTA 1, whose loads report to CTA 0, waits out the limit here)
                 for (int j = it > ST ? it - ST : 0; j < it; ++j) mbar_wait_clock(&full[j % ST], (j / ST) & 1);
+            } else if constexpr (PAIR) {
+                // The releases of the last min(it, ST) stages arrive here by
+                // CTA 0's commits, and no later load waits for them: this
+                // CTA's shared memory must outlive them.
+                for (int j = it > ST ? it - ST : 0; j < it && ok; ++j)
+                    ok = mbar_wait_clock(&empty[j % ST], (j / ST) & 1);
             }
         }
     } else if (warp == 1) {
@@ -404,16 +410,17 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         else tc::mma_bf16(acc, da, db, idesc, (kt | kk) != 0 ? 1u : 0u);
                     }
                     issued = true;
-                    if constexpr (PAIR) tc::mma_commit_pair(&empty[s]);
+                    if constexpr (PAIR) tc::mma_commit_pair(&empty[s], 3);
                     else tc::mma_commit(&empty[s]);
                 }
                 if (!ok) break;
-                if constexpr (PAIR) tc::mma_commit_pair(&acc_full[buf]);
+                if constexpr (PAIR) tc::mma_commit_pair(&acc_full[buf], 3);
                 else tc::mma_commit(&acc_full[buf]);
             }
             if (issued) {
-                // every MMA of this thread has completed once drain fires
-                if constexpr (PAIR) tc::mma_commit_pair(drain);
+                // every MMA of this thread has completed once drain fires (on
+                // CTA 0 of a pair alone: nothing in CTA 1 waits for it)
+                if constexpr (PAIR) tc::mma_commit_pair(drain, 1);
                 else tc::mma_commit(drain);
                 if (!mbar_wait_clock(drain, 0)) ok = false;
             }
@@ -610,7 +617,11 @@ k_gemm_bf16(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             ep.loss_partial[blockIdx.x] = l;
         }
     }
-    // neither CTA of a pair leaves while the other may signal it or use its operands
+    // Neither CTA of a pair leaves while the other may signal it or use its
+    // operands.  The barrier orders the threads' own arrivals (acc_empty); the
+    // tensor core's, which it does not order, have each been waited for where
+    // they land: empty by both producers, acc_full by both epilogues, drain by
+    // the issuer, and CTA 1's loads (on full) by the issuer.
     if constexpr (PAIR) tc::cluster_sync();
     if (warp == 1) {
         tc::fence_after_sync();

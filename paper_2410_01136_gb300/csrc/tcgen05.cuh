@@ -175,13 +175,13 @@ __device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, u
         ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// Arrive on the barrier at this offset in both CTAs when all previously issued
-// MMAs of this thread complete.
-__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+// Arrive on the barrier at this offset in the CTAs of `mask` (bit r: CTA r)
+// when all previously issued MMAs of this thread complete.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar, int mask) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
             smem_u32(bar)),
-        "h"((uint16_t)3)
+        "h"((uint16_t)mask)
         : "memory");
 }
 
