@@ -299,6 +299,12 @@ void synax_hmc_destroy(synax_hmc_t* hmc);
  * the caller zeroes it.  Exposed for tests of the kernel the surrogate runs. */
 int synax_gemm_bf16(const void* a_dev, int lda, const void* b_dev, int ldb, int M, int N, int K, float* c_dev,
                     int ldc, int* err_dev, void* stream);
+/* The tiles that a product of these sizes runs as on the current device
+ * (tests and diagnostics; no launch).  output: 0 FP32 (synax_gemm_bf16),
+ * 1 GELU, 2 GELU', 3 mean squared error.  *columns is the tile width, *pair 1
+ * where two CTAs share a tile of 256 rows (else 128 rows per CTA), *ctas the
+ * CTAs launched. */
+int synax_gemm_tile(int M, int N, int K, int output, int* columns, int* pair, int* ctas);
 
 /* synax_adjoint without a caller-provided workspace (the paper has no
  * counterpart: this is an interface for callers that cannot allocate device

@@ -151,6 +151,7 @@ SIGNATURES = {
     "synax_gemm_bf16": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_int,
                                        ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p,
                                        ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]),
+    "synax_gemm_tile": (ctypes.c_int, [ctypes.c_int] * 4 + [ctypes.POINTER(ctypes.c_int)] * 3),
     "synax_surrogate_create": (ctypes.c_int, [ctypes.POINTER(SynaxSurrogateCfg), ctypes.POINTER(_VP)]),
     "synax_surrogate_destroy": (None, [_VP]),
     "synax_surrogate_param_count": (ctypes.c_size_t, [_VP]),

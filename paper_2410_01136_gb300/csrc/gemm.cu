@@ -983,6 +983,18 @@ extern "C" int synax_gemm_bf16(const void* a_dev, int lda, const void* b_dev, in
     return gemm_bf16(a_dev, lda, b_dev, ldb, M, N, K, EPI_F32, ep, err_dev, (cudaStream_t)stream);
 }
 
+extern "C" int synax_gemm_tile(int M, int N, int K, int output, int* columns, int* pair, int* ctas) {
+    static const int epi[4] = {EPI_F32, EPI_BIAS_GELU, EPI_GELU_BWD, EPI_MSE};
+    if (!columns || !pair || !ctas || output < 0 || output > 3 || M < 1 || N < 1 || K < kGemmBK || K % kGemmBK != 0)
+        return SYNAX_EINVAL;
+    const int clusters = pair_clusters();
+    const GemmShape s = gemm_shape(M, N, K, epi[output], sm_count(), clusters);
+    *columns = s.bn;
+    *pair = s.pair ? 1 : 0;
+    *ctas = gemm_ctas(s, M, N, sm_count(), clusters);
+    return SYNAX_OK;
+}
+
 extern "C" int synax_wait_selftest(int* err_dev, long long* cycles_dev, void* stream) {
     if (!err_dev || !cycles_dev) return SYNAX_EINVAL;
     k_wait_selftest<<<1, 64, 0, (cudaStream_t)stream>>>(err_dev, cycles_dev, device_status_word());
