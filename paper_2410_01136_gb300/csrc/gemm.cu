@@ -679,13 +679,24 @@ __global__ void __launch_bounds__(64, 1) k_wait_selftest(int* err, long long* cy
 // narrower tiles on more SMs: 512 x 1024 x 9216 60.5 -> 44.2 us and 512 x 1024
 // x 1024 15.6 -> 11.0 us (32 columns, 128 tiles).  The order of summation
 // along K does not depend on the width.
+// With a long K and less than 128 KB of A, every CTA reads the same few L2
+// lines, whose slices then set the pace: halving stops at 64 CTAs
+// (48 from K = 8192: 1 x 2048 x 8192 43.6 us on 64, 41.1 on 32).  1 x 9216 x
+// 4096: 24.7 us on 36 CTAs, 31 on 72, 35 on 144; 1 x 4096 x 4096: 24.7 us on
+// 16, 23.0 on 64, 29 on 128; with 32 rows (256 KB) 144 CTAs take 23.0.  With a
+// short K (below 512 for a few rows, 1024 else) the epilogue decides, and
+// narrow tiles win: 1 x 9216 x 64 7.4 us on 36 CTAs, 6.1 on 144; x 512 8.4, 9.2.
 static int gemm_bn_for(int M, int N, int K, int sms) {
     int bn = (N >= 2048 || (N >= 1024 && K >= 4096)) ? 256 : (N >= 256 ? 128 : 64);
     auto cost = [&](int w) {
         const long long tiles = (long long)((N + w - 1) / w) * ((M + kGemmBM - 1) / kGemmBM);
         return (tiles + sms - 1) / sms * (kGemmBM + w);
     };
-    while (bn > 32 && cost(bn / 2) < cost(bn)) bn /= 2;
+    const bool few_lines = K >= (M < 8 ? 512 : 1024) && (long long)M * K < 65536;
+    while (bn > 32 && cost(bn / 2) < cost(bn)) {
+        if (few_lines && (N + bn / 2 - 1) / (bn / 2) > (K < 8192 ? 64 : 48)) break;
+        bn /= 2;
+    }
     return bn;
 }
 
@@ -713,7 +724,7 @@ static GemmShape gemm_shape(int M, int N, int K, int epi, int sms, int clusters)
     const bool f32_out = gemm_f32_out(epi);
     const long long rows = (M + kGemmBM - 1) / kGemmBM;
     if (f32_out && s.bn == 128 && N >= 1024 && rows * ((N + 255) / 256) >= 2LL * sms) s.bn = 256;
-    if (clusters > 0 && !f32_out && N >= 256 && K >= (epi == EPI_GELU_BWD ? 2048 : 1024)) {
+    if (clusters > 0 && !f32_out && rows > 1 && N >= 256 && K >= (epi == EPI_GELU_BWD ? 2048 : 1024)) {
         const long long tiles = rows * ((N + s.bn - 1) / s.bn);
         const long long pairs = (long long)((M + 255) / 256) * ((N + 255) / 256);
         if ((pairs + clusters - 1) / clusters * 256 < (tiles + sms - 1) / sms * (kGemmBM + s.bn)) s = {256, true};
