@@ -957,6 +957,10 @@ int gemm_tiles(int M, int N, int K) {
     return gemm_ctas(gemm_shape(M, N, K, EPI_MSE, sm_count(), clusters), M, N, sm_count(), clusters);
 }
 
+int gemm_columns(int M, int N, int K, int epi) {
+    return gemm_shape(M, N, K, epi, sm_count(), pair_clusters()).bn;
+}
+
 // C = A[M][K] . B[N][K]^T with the given epilogue.  A, B: BF16 row-major with
 // row pitches lda, ldb (elements); K a multiple of 64; pitches multiples of
 // 8; base pointers 16-byte aligned.

@@ -66,8 +66,11 @@ int device_sm_count();
 // calls it too).  Call before capturing a stream that will launch GEMMs.
 int gemm_init();
 
-// Number of CTAs of a GEMM of this shape (one loss partial each).
+// Number of CTAs of an EPI_MSE GEMM of this shape (one loss partial each).
 int gemm_tiles(int M, int N, int K);
+
+// Tile width of a GEMM of this shape and epilogue.
+int gemm_columns(int M, int N, int K, int epi);
 
 // Enqueue C = A . B^T with epilogue `epi` on `st`.  A [M][lda], B [N][ldb]
 // BF16 row-major, K a multiple of 64, pitches multiples of 8 elements, bases

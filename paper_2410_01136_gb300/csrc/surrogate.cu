@@ -1225,12 +1225,23 @@ int synax_surrogate(synax_surrogate_t* s, const float* theta_dev, int n, float* 
             return e == cudaSuccess ? SYNAX_OK : record_cuda_error((int)e);
         };
         if (vjp) SX_TRY(launch_seed());
+        // The first product's set-up overlaps the gather, so that its CTAs take
+        // the SMs before the seed's do.  A long seed (25 M elements: 150 MB,
+        // 22 us) must get there first: a CTA of 128 columns or more leaves no
+        // registers for the seed's beside it (168 x 320 + 64 x 256 > 65536), and
+        // a seed held to the few SMs left over is still running when the output
+        // layer's persistent CTAs need them.  7000 sets of width 256, 3072 basis
+        // rows: 298 us with the overlap, 252 without (5000 to 9000 sets: 236-341
+        // against 213-290); a shorter seed or a narrower tile gains from the
+        // overlap (3000 sets: 143 against 154).
+        const bool seed_first = vjp && (long long)m * s->n_out >= 3LL << 23 &&
+                                gemm_columns(m, s->N[0], s->K[0], EPI_BIAS_GELU) >= 128;
         GatherArgs a = gather_identity(s, theta_dev + (long long)r0 * nt, m, s->eX[0], nullptr, nullptr);
         k_gather_input<<<(m + 3) / 4, 128, 0, st>>>(a);
         SX_TRY(launch_status());
         for (int l = 0; l < L; ++l) {
             GemmEpiParams ep{};
-            ep.overlap = 1;
+            ep.overlap = l > 0 || !seed_first;
             ep.bias = s->b + s->boff[l];
             if (l < L - 1) {
                 ep.out_z = vjp ? s->eZ[l] : nullptr;
