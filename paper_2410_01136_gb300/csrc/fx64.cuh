@@ -204,6 +204,7 @@ SYNAX_FX_FN u64 rcp_core(u64 D) {
     // 24-bit seed r0 (Q0.32, < 1) from the FP32 reciprocal of the leading bits
     u32 s = rcp_seed(0x3F800000u | (u32)((D << 1) >> 41));
     s = s > 0x3F7FFFFFu ? 0x3F7FFFFFu : s;
+    s = s < 0x3F000000u ? 0x3F000000u : s;                  // in [1/2, 1)
     const u32 r0 = (s << 8) | 0x80000000u;
     const u32 Dh = (u32)(D >> 32), Dl = (u32)D;
     // e = 1 - d r0 in units of 2^-63, |e| < 2^42; 1/d = r0 (1 + e + e^2 + ...)
