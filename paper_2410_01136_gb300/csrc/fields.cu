@@ -28,7 +28,7 @@ k_eval_fields(const MapParams<R> P, const double* __restrict__ pos, const double
         const int base = grid_locate<R>(P, x, y, z, fx, fy, fz);
         grid_eval<R>(P, gc, base, fx, fy, fz, x, y, z, B, N0, ne, loc);
     } else {
-        Model<MODEL>::eval(P.m, s_arms, R(tdist[i]), x, y, z, ac, B, N0, ne, loc);
+        Model<MODEL>::template eval<R, FieldMath<R>>(P.m, s_arms, R(tdist[i]), x, y, z, ac, B, N0, ne, loc);
     }
     out[5 * i + 0] = (double)B[0];
     out[5 * i + 1] = (double)B[1];

@@ -15,11 +15,20 @@
 // at the same error against 64-bit values; CUDA's functions are specified to
 // 1 ulp.
 //
-// Accuracy: 62 to 63 correct bits before the final rounding, i.e. at most
-// 0.51 ulp, except that log and atan2 carry an absolute error of 2^-60 next
-// to their zeros.  Arguments outside each function's ordinary range
-// (non-normal, huge, zero or negative where that is special, NaN) go to the
-// CUDA function.
+// Accuracy: 60 to 63 correct bits before the final rounding, i.e. at most 0.53
+// ulp of the result, where division and square root round correctly in
+// hardware.  Beside a zero of the function:
+//  * log, atan2 and sincos (at non-zero multiples of pi/2) keep this relative
+//    accuracy with ZEROS (the default), and without it have an absolute error
+//    of 2^-60.  The march goes without (10 to 20 integer instructions per call):
+//    there these values enter sums, phases and products of order one.  Fields
+//    evaluated for the caller take ZEROS, as a component may be nothing but
+//    such a value;
+//  * the tanh of sech2_tanh and the weights of trilinear_weights have an
+//    absolute error of 2^-60 (formed in FP64 from e^-2x and from 1 - f they had
+//    2^-53).
+// Arguments outside each function's ordinary range (non-normal, huge, zero or
+// negative where that is special, NaN) go to the CUDA function.
 //
 // Method: the polynomials interpolate 2^f, atanh, sin, cos and atan at
 // Chebyshev nodes of the reduced range (computed in 400-bit arithmetic;
@@ -286,15 +295,19 @@ SYNAX_FX_FN double rsqrt(double x) {
     return pack(mul_1pg((u64)r0 << 31, g), -half - 63, 0);
 }
 
-// log2(m) for m = M in [1, 2): returns |l| (Q2.62) and neg, where
-// log2(m) = l, or 1 - |l| with up = 1, so that |l| <= 1/2.
-SYNAX_FX_FN u64 log2_core(u64 M, int& up) {
+// log2(m) for m = M in [1, 2): log2(m) = l, or 1 - l with up = 1, so that
+// 0 <= l <= 1/2.  Returns 2^lz l as Q2.62: lz normalises |m - 1| (or 2 - m) where
+// ZEROS, so that a small l keeps all its bits (else lz = 0).
+template <bool ZEROS>
+SYNAX_FX_FN u64 log2_core(u64 M, int& up, int& lz) {
     up = M > 0xB504F333F9DE6484ull;                           // m > sqrt 2: log2(m / 2) < 0
     const u64 a = up ? 0ull - M : M - 0x8000000000000000ull;   // |m - 1| or 2 - m, Q1.63
     const u64 D = (M >> 1) + (up ? 0x8000000000000000ull : 0x4000000000000000ull);
     // D is (m + 2)/2 or (m + 1)/2 in [1, 2); s = a / (2 D), Q0.64
     const u64 R = rcp_core(D);
-    const u64 s = mulhi(a, R) << 1;
+    lz = ZEROS ? clz(a) & 63 : 0;
+    const u64 sn = mulhi(a << lz, R) << 1;
+    const u64 s = sn >> lz;
     const u64 u = mh(s, s);
     u64 p = 0x0C3EC75D74CD7069ull;                            // (2 / ln 2) atanh(s) / s, Q2.62
     p = 0x0C3BA01CC4BFBA70ull + mh(p, u);
@@ -305,10 +318,10 @@ SYNAX_FX_FN u64 log2_core(u64 M, int& up) {
     p = 0x24EED8A1DF3F9890ull + mh(p, u);
     p = 0x3D8E13B87407F8C2ull + mh(p, u);
     p = 0xB8AA3B295C17F0BBull + mh(p, u);
-    return mh(s, p);
+    return mh(sn, p);
 }
 // ln x (NATURAL) or log2 x.
-template <bool NATURAL>
+template <bool NATURAL, bool ZEROS = true>
 SYNAX_FX_FN double log_any(double x) {
     const u64 b = bits_of(x);
     const int ex = biased_exp(b);
@@ -319,17 +332,17 @@ SYNAX_FX_FN double log_any(double x) {
         return NATURAL ? std::log(x) : std::log2(x);
 #endif
     }
-    int up;
-    const u64 l = log2_core(mantissa(b), up);
+    int up, lzl;
+    const u64 ln = log2_core<ZEROS>(mantissa(b), up, lzl);
     const int e = ex - 1023 + up;
-    // |log2 x| as v 2^k: l alone (Q2.62), or |e| +- l with as many fraction bits as |e| leaves
+    // |log2 x| as v 2^k: l alone (2^lzl l, Q2.62), or |e| +- l with as many fraction bits as |e| leaves
     const u32 ae = (u32)(e < 0 ? -e : e);
     const int sh = 64 - clz(ae);
-    const u64 ls = l >> sh;
+    const u64 ls = (ln >> lzl) >> sh;
     u64 v = ((u64)ae << (62 - sh)) + ((e < 0) == (up != 0) ? ls : 0ull - ls);
-    v = ae == 0 ? l : v;
+    v = ae == 0 ? ln : v;
     const u64 sign = (ae == 0 ? up != 0 : e < 0) ? 0x8000000000000000ull : 0ull;
-    int k = sh - 62;
+    int k = (ae == 0 ? -lzl : sh) - 62;
     if (NATURAL) {
         const int lz = clz(v);
         v = mulhi(v << (lz & 63), 0xB17217F7D1CF79ABull);       // ln 2, Q0.64
@@ -338,13 +351,23 @@ SYNAX_FX_FN double log_any(double x) {
     return pack(v, k, sign);
 }
 
+// The 64 bits below (hi:lo) >> s, s in [0, 128).
+SYNAX_FX_FN u64 below128(u64 hi, u64 lo, int s) {
+    const int t = s & 63;
+    const u64 w0 = s < 64 ? 0ull : lo, w1 = s < 64 ? lo : hi;
+    return (w0 >> t) | ((w1 << 1) << (63 - t));
+}
+
 // sin and cos of x radians, or (REV) of x revolutions.
-template <bool REV>
+template <bool REV, bool ZEROS = true>
 SYNAX_FX_FN void sincos_any(double x, double* sn, double* cs) {
     const u64 b = bits_of(x);
     const int ex = biased_exp(b);
-    // huge (2^30 radians; any fraction of 2^60 revolutions is exact here), subnormal or not finite
-    if (ex > 1023 + (REV ? 60 : 30) || (ex == 0 && (b << 1) != 0)) {
+    // Huge, subnormal or not finite.  The product with 4 / (2 pi) is off by up to 2^(e - 125) for
+    // |x| in [2^e, 2^(e + 1)), which below 2^14 radians is 2^-59.5 of the distance to the nearest
+    // multiple of pi/2 or less (29 pi/2 is 2^-60.5 from a double, and so its doubles in proportion).
+    // Any fraction of 2^60 revolutions is exact.
+    if (ex > 1023 + (REV ? 60 : (ZEROS ? 13 : 30)) || (ex == 0 && (b << 1) != 0)) {
 #ifdef __CUDACC__
         if (REV) ::sincospi(2.0 * x, sn, cs);
         else ::sincos(x, sn, cs);
@@ -398,7 +421,18 @@ SYNAX_FX_FN void sincos_any(double x, double* sn, double* cs) {
     pc = 0x4EF4F326F9177969ull - mh(pc, u);
     // an unreduced angle keeps its full mantissa (8 |x| = hi 2^(e4 + 3 - 63))
     const bool whole = quad == 0 && e4 < -3;
-    const double s0 = whole ? pack(mh(hi, ps), e4 + 3 - 63, rs << 63) : pack(mh(w, ps), -64, rs << 63);
+    u64 wn = w;                                               // 8 |r| 2^lz
+    int lz = 0;
+    if (ZEROS) {
+        // |r| with the 64 bits below it, normalised
+        const u64 rl = below128(hi, lo, 63 - e4);
+        const u64 h = rs ? ~r + (rl == 0 ? 1 : 0) : r, l = rs ? 0ull - rl : rl;
+        const u64 h1 = h ? h : l, l1 = h ? l : 0ull;
+        const int z = clz(h1);
+        wn = (h1 << (z & 63)) | ((l1 >> 1) >> ((63 - z) & 63));
+        lz = (h ? z : z + 64) - 3;
+    }
+    const double s0 = whole ? pack(mh(hi, ps), e4 + 3 - 63, rs << 63) : pack(mh(wn, ps), -64 - lz, rs << 63);
     const double c0 = pack(0x8000000000000000ull - (mh(u, pc) >> 1), -63, 0);
     const bool swap = quad & 1;
     const u64 ss = bits_of(swap ? c0 : s0) ^ ((u64)(quad >> 1) << 63) ^ (b & 0x8000000000000000ull);
@@ -408,6 +442,7 @@ SYNAX_FX_FN void sincos_any(double x, double* sn, double* cs) {
 }
 
 // atan2(y, x)
+template <bool ZEROS = true>
 SYNAX_FX_FN double atan2(double y, double x) {
     const u64 yb = bits_of(y), xb = bits_of(x);
     const u64 sign_bit = 0x8000000000000000ull;
@@ -415,7 +450,8 @@ SYNAX_FX_FN double atan2(double y, double x) {
     const bool steep = ya > xa;                               // |y| > |x| (the bits of FP64 magnitudes are ordered)
     const u64 big = steep ? ya : xa, small = steep ? xa : ya;
     const int eb = biased_exp(big), de = eb - biased_exp(small);
-    if (eb == 0 || eb == 0x7FF || (biased_exp(small) == 0 && small != 0)) {
+    // (a quotient that may fall below the normal range included)
+    if (eb == 0 || eb == 0x7FF || (small != 0 && (biased_exp(small) == 0 || (ZEROS && de > 1000)))) {
 #ifdef __CUDACC__
         return ::atan2(y, x);
 #else
@@ -455,7 +491,9 @@ SYNAX_FX_FN double atan2(double y, double x) {
     const u64 pi = 0xC90FDAA22168C234ull;                     // Q2.62
     t = steep ? (pi >> 1) - t : t;
     t = (xb & sign_bit) ? pi - t : t;
-    return pack(t, -62, yb & sign_bit);
+    // beside zero, from the quotient before its shift: q 2^-de atan(w) / w
+    const bool near0 = ZEROS && !steep && de >= 2 && !(xb & sign_bit);
+    return pack(near0 ? mulhi(q << 1, p) : t, -62 - (near0 ? de : 0), yb & sign_bit);
 }
 
 // sech^2 x and tanh x for 0 <= x < 300, from e = e^(-2x): 4 e / (1 + e)^2 and (1 - e) / (1 + e).

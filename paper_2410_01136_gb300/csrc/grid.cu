@@ -34,7 +34,7 @@ k_grid_sample(const MapParams<R> P, int nx, int ny, int nz, R hx, R hy, R hz, R*
         const ArmCoord<R> ac = arm_coord_direct<R>(x, y, M<R>::sqrt(x * x + y * y));
         R B[3], N0, ne;
         FieldLocal<R> loc;
-        Model<MODEL>::eval(P.m, s_arms, t, x, y, z, ac, B, N0, ne, loc);
+        Model<MODEL>::template eval<R, FieldMath<R>>(P.m, s_arms, t, x, y, z, ac, B, N0, ne, loc);
         out[3 * q + 0] = B[0];
         out[3 * q + 1] = B[1];
         out[3 * q + 2] = B[2];

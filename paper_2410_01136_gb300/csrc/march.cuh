@@ -167,10 +167,12 @@ template <> struct M<float> {
 };
 
 // FP64: the fixed-point functions of fx64.cuh in place of CUDA's, which run on
-// the FP64 pipe (2 lanes per clock and SM) that bounds this march.
+// the FP64 pipe (2 lanes per clock and SM) that bounds this march.  Logarithms,
+// atan2, pixel and field angles and phases with an absolute error of 2^-60 beside their
+// zeros, as they enter sums and phases of order one.
 template <> struct M<double> {
     static __device__ __forceinline__ double exp(double x) { return fx::exp_any<true>(x); }
-    static __device__ __forceinline__ double log(double x) { return fx::log_any<true>(x); }
+    static __device__ __forceinline__ double log(double x) { return fx::log_any<true, false>(x); }
     static __device__ __forceinline__ double div(double a, double b) { return fx::div(a, b); }
     static __device__ __forceinline__ double sqrt(double x) { return fx::sqrt(x); }
     static __device__ __forceinline__ double mulc(double x, double c) { return x * c; }
@@ -181,17 +183,29 @@ template <> struct M<double> {
     static __device__ __forceinline__ double rcp_shape(double x) { return fx::rcp(x); }
     static __device__ __forceinline__ double rsqrt_shape(double x) { return fx::rsqrt(x); }
     static __device__ __forceinline__ double mul_shape(double x, double c) { return x * c; }
-    static __device__ __forceinline__ double log2_fast(double x) { return fx::log_any<false>(x); }
+    static __device__ __forceinline__ double log2_fast(double x) { return fx::log_any<false, false>(x); }
     static __device__ __forceinline__ double rcp_fast(double x) { return fx::rcp(x); }
-    static __device__ __forceinline__ double atan2(double y, double x) { return fx::atan2(y, x); }
+    static __device__ __forceinline__ double atan2(double y, double x) { return fx::atan2<false>(y, x); }
     static __device__ __forceinline__ double floor(double x) { return ::floor(x); }
     static __device__ __forceinline__ double abs(double x) { return ::fabs(x); }
     static __device__ __forceinline__ double min(double a, double b) { return ::fmin(a, b); }
     static __device__ __forceinline__ double max(double a, double b) { return ::fmax(a, b); }
-    static __device__ __forceinline__ void sincos(double x, double* s, double* c) { fx::sincos_any<false>(x, s, c); }
-    static __device__ __forceinline__ void sincospi(double x, double* s, double* c) { fx::sincos_any<true>(0.5 * x, s, c); }
+    static __device__ __forceinline__ void sincos(double x, double* s, double* c) { fx::sincos_any<false, false>(x, s, c); }
+    static __device__ __forceinline__ void sincospi(double x, double* s, double* c) { fx::sincos_any<true, false>(0.5 * x, s, c); }
     // sin and cos of 2 pi r
-    static __device__ __forceinline__ void sincos_rev(double r, double* s, double* c) { fx::sincos_any<true>(r, s, c); }
+    static __device__ __forceinline__ void sincos_rev(double r, double* s, double* c) {
+        fx::sincos_any<true, false>(r, s, c);
+    }
+};
+
+// The traits of fields that are handed to the caller: logarithms, angles, sines
+// and cosines keep their relative accuracy beside their zeros (fx64.cuh), since
+// a field component may be nothing but such a value.
+template <typename R> struct FieldMath : M<R> {};
+template <> struct FieldMath<double> : M<double> {
+    static __device__ __forceinline__ double log(double x) { return fx::log_any<true>(x); }
+    static __device__ __forceinline__ double atan2(double y, double x) { return fx::atan2(y, x); }
+    static __device__ __forceinline__ void sincos(double x, double* s, double* c) { fx::sincos_any<false>(x, s, c); }
 };
 
 // ---------------------------------------------------------------------------
@@ -860,7 +874,7 @@ __device__ __forceinline__ void set_flat_z(FieldLocal<R>& loc, const FlatZ& fz) 
 template <int MODEL> struct Model;
 
 template <> struct Model<SYNAX_MODEL_TOY> {
-    template <typename R>
+    template <typename R, typename F = M<R>>
     static __device__ __forceinline__ void eval(const R* m, const R* /*arms*/, R t, R /*x*/, R /*y*/,
                                                 R /*z*/, const ArmCoord<R>& /*ac*/, R B[3], R& N0,
                                                 R& ne, FieldLocal<R>& /*loc*/) {
@@ -874,11 +888,10 @@ template <> struct Model<SYNAX_MODEL_TOY> {
 };
 
 template <> struct Model<SYNAX_MODEL_WMAP> {
-    template <typename R>
+    template <typename R, typename F = M<R>>
     static __device__ __forceinline__ void eval(const R* m, const R* /*arms*/, R /*t*/, R x, R y, R z,
                                                 const ArmCoord<R>& /*ac*/, R B[3], R& N0, R& ne,
                                                 FieldLocal<R>& loc) {
-        using F = M<R>;
         const R rho2 = x * x + y * y;
         const bool has_rho = rho2 > R(0);
         const R rho = F::sqrt(rho2);
@@ -919,11 +932,10 @@ template <> struct Model<SYNAX_MODEL_WMAP> {
 };
 
 template <> struct Model<SYNAX_MODEL_JF12> {
-    template <typename R>
+    template <typename R, typename F = M<R>>
     static __device__ __forceinline__ void eval(const R* m, const R* arms, R /*t*/, R x, R y, R z,
                                                 const ArmCoord<R>& ac, R B[3], R& N0, R& ne,
                                                 FieldLocal<R>& loc) {
-        using F = M<R>;
         const R rho2 = x * x + y * y;
         const bool has_rho = rho2 > R(0);
         // correctly rounded rho: it enters the RM through n_e and the field
@@ -1015,11 +1027,10 @@ template <> struct Model<SYNAX_MODEL_JF12> {
 // accurate one (logf, sincosf, expf).
 
 template <> struct Model<SYNAX_MODEL_WMAP_STACK> {
-    template <typename R>
+    template <typename R, typename F = M<R>>
     static __device__ __forceinline__ void eval(const R* m, const R* /*arms*/, R /*t*/, R x, R y, R z,
                                                 const ArmCoord<R>& /*ac*/, R B[3], R& N0, R& ne,
                                                 FieldLocal<R>& loc) {
-        using F = M<R>;
         const R rho2 = x * x + y * y;
         const bool has_rho = rho2 > R(0);
         const R rho = F::sqrt(rho2);
