@@ -27,6 +27,10 @@ k_eval_fields(const MapParams<R> P, const double* __restrict__ pos, const double
         R fx, fy, fz;
         const int base = grid_locate<R>(P, x, y, z, fx, fy, fz);
         grid_eval<R>(P, gc, base, fx, fy, fz, x, y, z, B, N0, ne, loc);
+        // a NaN position has no cell (it is clamped to the first): FP64's weights,
+        // fixed-point fractions, would not carry it
+        const R f = fx + fy + fz;
+        if (f != f) B[0] = B[1] = B[2] = f;
     } else {
         Model<MODEL>::template eval<R, FieldMath<R>>(P.m, s_arms, R(tdist[i]), x, y, z, ac, B, N0, ne, loc);
     }

@@ -532,7 +532,7 @@ SYNAX_FX_FN double split_floor(double v, int& whole) {
     f = neg ? 0ull - f : f;
     return pack(f, -64, 0);
 }
-// f in [0, 1] as Q1.63.
+// f in [0, 1] as Q1.63 (a number: NaN has no fixed-point form).
 SYNAX_FX_FN u64 unit_q63(double f) {
     const u64 b = bits_of(f);
     const int s = 1023 - biased_exp(b);
