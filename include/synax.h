@@ -523,9 +523,11 @@ int synax_surrogate_load(synax_surrogate_t* s, const char* path);
  * one ray, 8, 16 or 32.  lanes = 0 restores the built-in rule.  With
  * n_steps_min >= 0 the value applies to maps whose step count falls in the
  * tuning bin containing n_steps_min (bins edges 64, 128, 256, ..., 4096);
- * with n_steps_min < 0 it is forced for every map.  Results do not depend on
- * the choice beyond rounding; the autotuner (paper_2410_01136_gb300/tune.py)
- * measures the candidates and installs the fastest.  Process-wide setting. */
+ * with n_steps_min < 0 it is forced for every map.  FP32 marches and batches
+ * only: SYNAX_F64 maps take 16 lanes from 1216 rays, else 32, whatever is set
+ * here.  Results do not depend on the choice beyond rounding; the autotuner
+ * (paper_2410_01136_gb300/tune.py) measures the candidates and installs the
+ * fastest.  Process-wide setting. */
 int synax_set_lanes_per_ray(int n_steps_min, int lanes);
 
 /* ---- device status word (no counterpart in the paper) ----

@@ -394,7 +394,8 @@ def set_batch_pairing(on: bool) -> None:
 
 def set_lanes_per_ray(lanes: int, n_steps_min: int = -1) -> None:
     """Launch tuning: 8, 16 or 32 lanes per ray (0 = built-in rule), for every
-    map (n_steps_min < 0) or for the step-count bin containing n_steps_min."""
+    FP32 map (n_steps_min < 0) or for the step-count bin containing
+    n_steps_min.  FP64 maps have a rule of their own (synax_set_lanes_per_ray)."""
     check(lib().synax_set_lanes_per_ray(int(n_steps_min), int(lanes)), "synax_set_lanes_per_ray")
 
 

@@ -43,7 +43,9 @@ int lanes_per_ray(int n_steps, long long n_pix) {
 // grid map of Nside 64, 512 steps 4.18, 4.03, 4.02 ms; JF12-type map of
 // Nside 64, 200 steps 4.35, 3.94, 3.83 ms; WMAP-type map of Nside 16, 128
 // steps 0.122, 0.106, 0.169 ms; JF12-type map + gradient of Nside 16, 100
-// steps 0.902, 0.783, 1.027 ms.
+// steps 0.902, 0.783, 1.027 ms.  8 lanes would gain up to 3 % at Nside 64 and
+// cost up to 60 % at Nside 16; they are not built, for half as many kernels again.
+// 1216 rays are 8 (a CTA's) on each of the 152 SMs.
 int lanes_per_ray_f64(long long n_pix) { return n_pix >= 8LL * 152 ? 16 : 32; }
 
 }  // namespace synax
