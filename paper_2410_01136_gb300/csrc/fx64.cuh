@@ -31,9 +31,10 @@
 // negative where that is special, NaN) go to the CUDA function.
 //
 // Method: the polynomials interpolate 2^f, atanh, sin, cos and atan at
-// Chebyshev nodes of the reduced range (computed in 400-bit arithmetic;
-// truncation below 2^-64 of the result); the reciprocal and the reciprocal
-// square root are Newton's from a 22-bit FP32 seed with one second-order step.
+// Chebyshev nodes of the reduced range (in 400-bit arithmetic, each coefficient
+// cut to its word; the interpolation is off by less than 2^-64 of the result);
+// the reciprocal and the reciprocal square root are a 22-bit FP32 seed and one
+// Newton-Raphson step with its second-order term.
 // Qa.b below: an unsigned 64-bit word whose unit is 2^-b.
 #pragma once
 
