@@ -227,8 +227,9 @@ def problem_struct(prob) -> SynaxProblem:
     s.r_max_kpc = float(prob.r_max_kpc)
     # slices: one C loop each (element by element the struct took twice as long,
     # a third of a small map's time)
-    s.box_kpc[:] = [float(v) for v in prob.box_kpc[:3]]
-    s.obs_kpc[:] = [float(v) for v in prob.obs_kpc[:3]]
+    box, obs = prob.box_kpc, prob.obs_kpc
+    s.box_kpc[:] = [float(box[0]), float(box[1]), float(box[2])]
+    s.obs_kpc[:] = [float(obs[0]), float(obs[1]), float(obs[2])]
     freqs = [float(f) for f in prob.freq_hz]
     if len(freqs) > MAX_FREQ:
         raise ValueError(f"at most {MAX_FREQ} frequencies")
