@@ -713,7 +713,7 @@ static int gemm_bn_for(int M, int N, int K, int sms) {
 // K = 1024 (16384 x 1024 x 1024: 47.7 against 52.6 us; K = 64: 39.4 against
 // 32.7), GELU' from 2048 (16384 x 1024 x 9216: 197 against 216 us; x 1024,
 // where its pre-activation is read in the epilogue: 54 against 50), MSE as
-// GELU.  FP32 outputs gain nothing: their stores bound them (16384 x 9216 x
+// GELU; no K between these was measured.  FP32 outputs gain nothing: their stores bound them (16384 x 9216 x
 // 1024: 217 against 219 us as pairs, x 64 124 against 91).
 struct GemmShape {
     int bn;
